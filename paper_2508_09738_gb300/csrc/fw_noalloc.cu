@@ -82,49 +82,139 @@ k_na_degrees(int64_t n, int64_t nnz, const int32_t* __restrict__ rp,
     }
 }
 
+// One row's energy from its products s_k = sum_j w_ij u_jk, k in steps of `ks`.
+__device__ __forceinline__ double na_row_energy(int K, const double* __restrict__ ui,
+                                                const double* s, int ks, double di, int f,
+                                                double inv_eps, double omega0, int comb) {
+    double quad = 0.0, pen = 0.0, fidt = 0.0;
+    for (int k = 0; k < K; ++k) {
+        const double u = ui[k];
+        const double lu = (comb ? di : 1.0) * u - s[k * ks];
+        quad += u * lu;
+        pen += u * (1.0 - u);
+        if (f >= 0) {
+            const double dlt = (k == f ? 1.0 : 0.0) - u;
+            fidt += dlt * dlt;
+        }
+    }
+    return 0.5 * quad + inv_eps * pen + (f >= 0 ? 0.5 * omega0 * fidt : 0.0);
+}
+
+// Entries of a warp's 32 rows normalised at a time.
+constexpr int kNaChunk = 256;
+// Dynamic shared memory of one warp: the chunk's weights and columns, the
+// rows' products.
+__host__ __device__ inline size_t na_warp_smem(int K) {
+    return size_t(kNaChunk) * (sizeof(double) + sizeof(int32_t)) + size_t(32) * K * sizeof(double);
+}
+
 // Per row i (FP64): 1/2 sum_k u_ik (L u)_ik + 1/eps sum_k u_ik (1 - u_ik)
 // + 1/2 omega_i sum_k (uhat_ik - u_ik)^2, with (L u)_ik = u_ik - sum_j
 // w_ij u_jk / sqrt(d_i d_j) (L_s) or d_i u_ik - sum_j w_ij u_jk (L = D - W).
 // Threads add their rows in order; the block adds its threads in a fixed
 // order and adds its total into the exact fixed-point accumulator, so the
 // result does not depend on the order in which blocks finish.
+//
+// FP64 issue bounds this kernel (an FP64 instruction holds a scheduler for 64
+// cycles; a square root and a division are about 35 of them), so every entry
+// is normalised once, not once per class, and by the next free lane: a warp
+// takes the contiguous entries of its 32 rows kNaChunk at a time, its lanes
+// normalise 32 entries together whatever rows they belong to, then take one
+// (row, class) each and add that row's entries of the chunk in CSR order (the
+// sums of one thread per row, in the same order).  300,007 rows, 14 entries
+// each, K = 6: 310 us a call, 1,720 us with the square root and the division
+// per entry and class and one thread per row.
 __global__ void __launch_bounds__(kBlock)
 k_na_energy(int64_t n, int64_t nnz, int K, const int32_t* __restrict__ rp,
             const int32_t* __restrict__ col, const double* __restrict__ w,
             const double* __restrict__ deg, const double* __restrict__ U, int64_t ldu,
             const int32_t* __restrict__ labels, double inv_eps, double omega0, int comb,
             unsigned long long* acc) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ int32_t s_rp[kBlock / 32][33];
+    __shared__ double s_deg[kBlock];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double* const sw = reinterpret_cast<double*>(smraw + warp * na_warp_smem(K));
+    double* const ss = sw + kNaChunk;                              // [32][K]
+    int32_t* const sc = reinterpret_cast<int32_t*>(ss + 32 * K);   // columns, -1: out of range
     const int64_t stride = int64_t(gridDim.x) * kBlock;
     double e_thr = 0.0;
-    for (int64_t i = blockIdx.x * int64_t(kBlock) + threadIdx.x; i < n; i += stride) {
-        const int64_t e0 = rp[i], e1 = rp[i + 1];
-        const double di = deg[i];
-        if (e0 < 0 || e1 > nnz || e1 < e0 || !(di > 0.0)) continue;  // flagged by k_na_degrees
-        int f = labels ? labels[i] : -1;
-        if (f < -1 || f >= K) {
-            atomicOr(&acc[kNaErrWord], kNaBadLabel);
-            f = -1;
+    for (int64_t i0 = blockIdx.x * int64_t(kBlock) + (threadIdx.x & ~31); i0 < n; i0 += stride) {
+        const int64_t i = i0 + lane;
+        const bool in = i < n;
+        const int32_t e0 = in ? rp[i] : 0, e1 = in ? rp[i + 1] : 0;
+        const double di = in ? deg[i] : 0.0;
+        const bool ok = in && !(e0 < 0 || e1 > nnz || e1 < e0 || !(di > 0.0));   // else flagged by k_na_degrees
+        int f = -1;
+        if (ok && labels) {
+            f = labels[i];
+            if (f < -1 || f >= K) {
+                atomicOr(&acc[kNaErrWord], kNaBadLabel);
+                f = -1;
+            }
         }
-        const double* ui = U + i * ldu;
-        double quad = 0.0, pen = 0.0, fidt = 0.0;
-        for (int k = 0; k < K; ++k) {
-            double s = 0.0;
-            for (int64_t e = e0; e < e1; ++e) {
+        if (!__all_sync(0xffffffffu, ok || !in)) {
+            // a flagged row: the call fails, whatever the energy; rows one by one
+            if (ok) {
+                for (int k = 0; k < K; ++k) {
+                    double s = 0.0;
+                    for (int32_t e = e0; e < e1; ++e) {
+                        const int32_t j = col[e];
+                        if (j < 0 || j >= n) continue;
+                        const double wij = comb ? w[e] : w[e] / sqrt(di * deg[j]);
+                        s += wij * U[j * ldu + k];
+                    }
+                    ss[lane * K + k] = s;
+                }
+                e_thr += na_row_energy(K, U + i * ldu, ss + lane * K, 1, di, f, inv_eps, omega0, comb);
+            }
+            __syncwarp();
+            continue;
+        }
+        const int rows = __popc(__ballot_sync(0xffffffffu, in));
+        s_rp[warp][lane] = e0;
+        if (lane == rows - 1) s_rp[warp][rows] = e1;
+        s_deg[threadIdx.x] = di;
+        for (int k = 0; k < K; ++k) ss[lane * K + k] = 0.0;
+        __syncwarp();
+        const int32_t* const q = s_rp[warp];
+        const int64_t last = q[rows];
+        for (int64_t b = q[0]; b < last; b += kNaChunk) {
+            const int cnt = last - b < kNaChunk ? int(last - b) : kNaChunk;
+            for (int t = lane; t < cnt; t += 32) {
+                const int64_t e = b + t;
                 const int32_t j = col[e];
-                if (j < 0 || j >= n) continue;
-                const double wij = comb ? w[e] : w[e] / sqrt(di * deg[j]);
-                s += wij * U[j * ldu + k];
+                const bool good = j >= 0 && j < n;
+                double v = w[e];
+                if (!comb && good) {
+                    int lo = 0, hi = rows - 1;   // the row that holds e
+                    while (lo < hi) {
+                        const int mid = (lo + hi + 1) >> 1;
+                        if (q[mid] <= e) lo = mid;
+                        else hi = mid - 1;
+                    }
+                    v = v / sqrt(s_deg[(threadIdx.x & ~31) + lo] * deg[j]);
+                }
+                sw[t] = v;
+                sc[t] = good ? j : -1;
             }
-            const double u = ui[k];
-            const double lu = (comb ? di : 1.0) * u - s;
-            quad += u * lu;
-            pen += u * (1.0 - u);
-            if (f >= 0) {
-                const double dlt = (k == f ? 1.0 : 0.0) - u;
-                fidt += dlt * dlt;
+            __syncwarp();
+            for (int t = lane; t < rows * K; t += 32) {
+                const int r = t / K, k = t - r * K;
+                const int a0 = q[r] > b ? int(q[r] - b) : 0;
+                const int a1 = q[r + 1] - b < cnt ? int(q[r + 1] - b) : cnt;
+                double s = ss[t];
+                for (int x = a0; x < a1; ++x) {
+                    const int32_t j = sc[x];
+                    if (j >= 0) s += sw[x] * U[j * ldu + k];
+                }
+                ss[t] = s;
             }
+            __syncwarp();
         }
-        e_thr += 0.5 * quad + inv_eps * pen + (f >= 0 ? 0.5 * omega0 * fidt : 0.0);
+        if (in)
+            e_thr += na_row_energy(K, U + i * ldu, ss + lane * K, 1, di, f, inv_eps, omega0, comb);
+        __syncwarp();
     }
     const double v[1] = {e_thr};
     block_accumulate<double, 1>(v, acc, 0, int(blockIdx.x % kAccCopies));
@@ -241,7 +331,11 @@ extern "C" fw_status fw_energy_noalloc(int64_t n, int32_t K, const int32_t* row_
     const int blocks = int(want < kNaMaxBlocks ? want : kNaMaxBlocks);
     k_na_degrees<<<blocks, kBlock, 0, s>>>(n, nnz, row_ptr_dev, col_dev, w_dev, deg, acc);
     FW_CUDA(cudaGetLastError());
-    k_na_energy<<<blocks, kBlock, 0, s>>>(n, nnz, K, row_ptr_dev, col_dev, w_dev, deg, U_dev,
+    const size_t smem = size_t(kBlock / 32) * na_warp_smem(K);
+    if (smem > 48 * 1024)   // K > 12: beyond what a kernel gets without asking
+        FW_CUDA(cudaFuncSetAttribute(k_na_energy, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     int(smem)));
+    k_na_energy<<<blocks, kBlock, smem, s>>>(n, nnz, K, row_ptr_dev, col_dev, w_dev, deg, U_dev,
                                           ldu, labels_dev, std::isinf(eps) ? 0.0 : 1.0 / eps,
                                           omega0, laplacian == FW_LAPLACIAN_COMB ? 1 : 0, acc);
     FW_CUDA(cudaGetLastError());
