@@ -113,7 +113,9 @@ typedef struct fw_seg fw_seg;
  * needs an FP32 iterate, K <= 16, 1, 2 or 4 lanes per row, n <= 311,296 and
  * the array plus the bins within one block's shared memory (n <= 280,574
  * for 8 < K <= 10 with 2 lanes), else the direct form runs.  Both forms give the
- * same bits.  FW_TABLE_OFF always runs the direct form. */
+ * same bits.  FW_TABLE_OFF always runs the direct form.  Under either of the
+ * two, fw_seg_solve runs that pass B also where it would run the resident
+ * kernel under FW_TABLE_AUTO. */
 enum { FW_TABLE_AUTO = 0, FW_TABLE_OFF = 1, FW_TABLE_ON = 2 };
 
 /* Fill *opts with defaults: eps 50, omega0 1000 (the paper's network values,
@@ -142,13 +144,19 @@ fw_status fw_seg_create(fw_seg **out, int64_t n, const int32_t *row_ptr_host,
  * g_k <= 0 (stationary, FW_OK), g_k <= tolerance (FW_OK), or max_iters updates
  * (FW_NOT_CONVERGED).  The test is made before the update, as in step 4 of
  * Alg. 3.  stats may be NULL.  Errors: FW_ERR_NUMERIC, FW_ERR_CUDA.
- * Execution: iterations run as a CUDA graph of iters_per_launch iterations
+ * Execution: problems of up to 311,296 rows and K <= 16 whose state fits the
+ * chip (class_table left at FW_TABLE_AUTO) run in one launch of the resident
+ * kernel: U and L U stay in registers from the first iteration to the last,
+ * on one thread-block cluster or on a cooperative grid of one block per SM at
+ * most.  Others run as a CUDA graph of iters_per_launch iterations
  * (2 kernels each, the step decision of each iteration taken at the start of
  * the next one, one finishing kernel per graph), launched repeatedly with one
  * launch queued ahead of the host's state check; fewer than iters_per_launch
  * remaining iterations run as direct launches of the same kernels.  With
  * refresh_every > 0, or on a stream that cannot be captured, the host checks
- * the state after every launch.  The stream is synchronised on return. */
+ * the state after every launch.  Both forms give the same bits.  The stream
+ * is synchronised on return.  FW_ERR_TIMEOUT: a wait inside the resident
+ * kernel ran out of its 2 s. */
 fw_status fw_seg_solve(fw_seg *h, fw_seg_stats *stats);
 
 /* Run at most `iters` iterations (fewer if the stop rule holds first) and
@@ -205,9 +213,10 @@ fw_status fw_seg_reset(fw_seg *h);
 /* Measurement of the iteration kernels in the form fw_seg_solve runs them
  * (each time is taken with two CUDA events on the handle's stream around one
  * captured graph, so no event sits between kernels):
- *   *ms_per_iter  a graph of `iters` (1..4096) fused iterations (pass A with
- *                 the previous iteration's step decision, pass B) and one
- *                 finishing kernel, divided by iters;
+ *   *ms_per_iter  a graph of `iters` (1..4096) iterations as the solve runs
+ *                 them, divided by iters: one resident launch, or pass A with
+ *                 the previous iteration's step decision and pass B per
+ *                 iteration and one finishing kernel;
  *   *ms_row_pass  a graph of `iters` launches of the fused pass A (update,
  *                 step decision, gradient, GLMO, gap pieces), per launch;
  *   *ms_csr_pass  a graph of `iters` launches of pass B (one-hot L S,

@@ -261,16 +261,21 @@ __device__ __forceinline__ bool last_to_arrive(uint32_t* cnt, uint32_t total) {
 // whatever the order of the atomic operations.  A problem has at most
 // kTilesTarget (< 2^11) tiles, so a total of values below 2^52 cannot
 // overflow the signed high word.  Non-finite or larger values raise *flag.
+__device__ __forceinline__ bool fx_split(double v, unsigned long long& lo, unsigned long long& hi) {
+    if (!isfinite(v) || fabs(v) >= 0x1p52) return false;
+    const double fl = floor(v);
+    lo = __double2ull_rz(ldexp(v - fl, 64));
+    hi = static_cast<unsigned long long>(__double2ll_rz(fl));
+    return true;
+}
 __device__ __forceinline__ void fx_add(unsigned long long* slot, unsigned long long* flag,
                                        double v) {
     static_assert(kTilesTarget < 2048, "fixed-point totals assume < 2^11 tiles");
-    if (!isfinite(v) || fabs(v) >= 0x1p52) {
+    unsigned long long lo, hi;
+    if (!fx_split(v, lo, hi)) {
         atomicOr(flag, 1ull);
         return;
     }
-    const double fl = floor(v);
-    const unsigned long long lo = __double2ull_rz(ldexp(v - fl, 64));
-    const unsigned long long hi = static_cast<unsigned long long>(__double2ll_rz(fl));
     const unsigned long long old = atomicAdd(&slot[0], lo);
     const unsigned long long carry = (old + lo < old) ? 1ull : 0ull;
     atomicAdd(&slot[1], hi + carry);
@@ -534,20 +539,153 @@ __device__ __forceinline__ StepCfg step_cfg(const ProbDesc& pd) {
 
 static_assert(kAccCopies == 1, "warp_decide reads one accumulator copy");
 
+__device__ __forceinline__ bool finite_bits(double v) {
+    return ((static_cast<unsigned long long>(__double_as_longlong(v)) >> 52) & 0x7ffull) != 0x7ffull;
+}
+__device__ __forceinline__ bool positive_bits(double v) {   // v > 0 for a v that is not NaN
+    return __double_as_longlong(v) > 0;
+}
+
+// A Q64.64 number as a double.  An FP64 instruction holds the scheduler for 64
+// cycles on GB300, so scalings by powers of two and tests work on the bits.
+__device__ __forceinline__ double fx_double(unsigned long long lo, unsigned long long hi) {
+    unsigned long long fb = static_cast<unsigned long long>(__double_as_longlong(double(lo)));
+    if (fb) fb -= 64ull << 52;   // lo 2^-64
+    return double(static_cast<long long>(hi)) + __longlong_as_double(static_cast<long long>(fb));
+}
+
+// The step along D for gap g > 0 and curvature q (finite): the exact line
+// search of eq. 10, or Armijo halving.
+__device__ __forceinline__ double step_length(double g, double q, int step_rule) {
+    double a = 1.0;
+    if (positive_bits(q)) {
+        const double r = g / q;   // one division serves both rules; r >= 0
+        if (step_rule == 0) {
+            a = __double_as_longlong(r) < __double_as_longlong(1.0) ? r : 1.0;
+        } else {
+            // Armijo: largest 0.5^j with E(U) - E(U + a D) = a g - a^2 q / 2 >= 1e-6 a g,
+            // i.e. a <= 2 (1 - 1e-6) g / q
+            const double amax = 2.0 * (1.0 - 1e-6) * r;
+            for (int j = 0; j < 1100 && a > amax; ++j) a *= 0.5;
+        }
+    }
+    return a;
+}
+
+// <D, H D> from <D,LS>, <D,LU>, sum w||D||^2 and ||D||^2.
+__device__ __forceinline__ double curvature(double pLS, double tLU, double nW, double nD,
+                                            double inv_eps) {
+    return __fma_rn(-2.0 * inv_eps, nD, (pLS - tLU) + nW);
+}
+
+// E(U + a D) = E - a g + a^2 q / 2.
+__device__ __forceinline__ double next_energy(double E, double g, double q, double a) {
+    return __fma_rn(0.5 * a * a, q, __fma_rn(-a, g, E));
+}
+
+// A step decision: the same in every lane, except Sq.
+struct Decision {
+    double Sq;   // lane 2q: quantity q of the iteration
+    double g, g0, q, a;
+    int status, done;
+};
+
 // The step decision of one iteration, taken by one warp (all 32 lanes call
 // it) from the iteration's totals S = (g, ||D||^2, sum w||D||^2, <D,LU>, |I|,
-// <D,LS>) in accumulator bank `accb` and the inputs in[c]: the stop test of
-// Alg. 3 step 4, then the curvature q = <D, H D> and the step (exact line
-// search, eq. 10, or Armijo halving).
-//
+// <D,LS>) and the inputs in: the stop test of Alg. 3 step 4, then the
+// curvature q = <D, H D> and the step (exact line search, eq. 10, or Armijo
+// halving).  Word l < kAccWords of the totals (Q64.64 pairs, then the
+// non-finite flag) is in lane l's w; lane 2q turns quantity q into a double.
+__device__ __forceinline__ Decision decide(unsigned long long w, const StepIn& in, int err,
+                                           const StepCfg& cfg) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    // Q64.64 (lo word in lane 2q, hi in 2q+1) -> double
+    double Sq = fx_double(w, __shfl_down_sync(full, w, 1));
+    if (__shfl_sync(full, w, kAccFlag) != 0ull && lane == 0) Sq = CUDART_NAN;
+    const bool bad = (lane == 0 || lane == 2 || lane == 4 || lane == 6 || lane == 10) && !finite_bits(Sq);
+    const bool nonfinite = __any_sync(full, bad);
+    const double g = __shfl_sync(full, Sq, 0);
+    const int active = int(__shfl_sync(full, Sq, 8));
+    const double q = curvature(__shfl_sync(full, Sq, 10), __shfl_sync(full, Sq, 6),
+                               __shfl_sync(full, Sq, 4), __shfl_sync(full, Sq, 2), cfg.inv_eps);
+    const double g0 = in.g0_set ? in.g0 : g;
+    int status = 2;  // FW_PENDING
+    int done = 0;
+    if (err) {
+        status = -7;  // FW_ERR_TIMEOUT
+        done = 1;
+    } else if (nonfinite) {
+        status = -6;  // FW_ERR_NUMERIC
+        done = 1;
+    } else if (active == 0 || !positive_bits(g)) {   // g is finite here
+        status = 0;
+        done = 1;
+    } else if (positive_bits(cfg.gap_tol) && g <= (cfg.tol_mode ? cfg.gap_tol * g0 : cfg.gap_tol)) {
+        status = 0;
+        done = 1;
+    } else if (in.iter >= cfg.max_iters) {
+        status = 1;  // FW_NOT_CONVERGED
+        done = 1;
+    } else if (!finite_bits(q)) {
+        status = -6;
+        done = 1;
+    }
+    const double a = done ? 1.0 : step_length(g, q, cfg.step_rule);
+    return Decision{Sq, g, g0, q, a, status, done};
+}
+
+// The inputs of the next decision after decision d on inputs `in`.
+__device__ __forceinline__ StepIn next_in(const StepIn& in, const Decision& d) {
+    StepIn nx;
+    nx.E = in.E;
+    nx.g0 = d.g0;
+    nx.iter = in.iter;
+    nx.g0_set = 1;
+    if (!d.done) {
+        nx.E = next_energy(in.E, d.g, d.q, d.a);
+        nx.iter = in.iter + 1;
+    }
+    return nx;
+}
+
+// Write decision d into the state: each statistic from its lane, the rest
+// from lane 0, the next decision's inputs into in[slot] included; q and alpha
+// keep their last values once done.
+__device__ __forceinline__ void commit_decision(ProbState* st, const Decision& d, const StepIn& nx,
+                                                int slot) {
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) st->g = d.Sq;
+    if (lane == 2) st->nD = d.Sq;
+    if (lane == 4) st->nW = d.Sq;
+    if (lane == 6) st->tLU = d.Sq;
+    if (lane == 8) st->active = int(d.Sq);
+    if (lane == 10) st->pLS = d.Sq;
+    if (lane == 0) {
+        st->g0 = d.g0;
+        st->g0_set = 1;
+        st->status = d.status;
+        st->done = d.done;
+        if (!d.done) {
+            st->q = d.q;
+            st->alpha = d.a;
+            st->alpha_f = float(d.a);
+        }
+        st->has_update = d.done ? 0 : 1;
+        st->E = nx.E;
+        st->iter = nx.iter;
+        st->in[slot] = nx;
+    }
+}
+
+// The decision on the totals in accumulator bank `accb` and the inputs in[c].
 // Lane l loads word l of the bank; lanes 16..19 load in[c] and the error
-// flag, so everything arrives in one round trip, and lane 2q turns quantity
-// q into a double.  Spread this way the decision needs few registers per
-// thread, which matters where it is fused into pass A.  With `commit` the
-// warp writes the result into the state (each statistic from its lane, the
-// rest from lane 0), in[c ^ 1] included; q and alpha keep their last values
-// once done.  k_finish, pass A (fused) and the persistent kernel's last block
-// all run this code, so their decisions agree bit for bit.
+// flag, so everything arrives in one round trip.  Spread this way the
+// decision needs few registers per thread, which matters where it is fused
+// into pass A.  With `commit` the warp writes the result into the state, in[c
+// ^ 1] included.  k_finish, pass A (fused) and the persistent kernel's last
+// block all run this code, and the resident kernel decide() on its own
+// totals, so their decisions agree bit for bit.
 // Returns `done` in every lane; *alpha = the step.
 __device__ __forceinline__ int warp_decide(const unsigned long long* accb, ProbState* st, int c,
                                            const StepCfg& cfg, bool commit, double* alpha) {
@@ -558,89 +696,17 @@ __device__ __forceinline__ int warp_decide(const unsigned long long* accb, ProbS
     if (lane < kAccWords) w = __ldcg(accb + lane);
     else if (lane >= 16 && lane < 19) w = __ldcg(inw + (lane - 16));
     else if (lane == 19) w = static_cast<unsigned long long>(static_cast<unsigned>(__ldcg(&st->err)));
-    // Q64.64 (lo word in lane 2q, hi in 2q+1) -> double
-    const unsigned long long hw = __shfl_down_sync(full, w, 1);
-    double Sq = double(static_cast<long long>(hw)) + ldexp(double(w), -64);
-    if (__shfl_sync(full, w, kAccFlag) != 0ull && lane == 0) Sq = CUDART_NAN;
-    const bool bad = (lane == 0 || lane == 2 || lane == 4 || lane == 6 || lane == 10) && !isfinite(Sq);
-    const bool nonfinite = __any_sync(full, bad);
-    const double g = __shfl_sync(full, Sq, 0);
-    const int active = int(__shfl_sync(full, Sq, 8));
-    const double qL = __shfl_sync(full, Sq, 10) - __shfl_sync(full, Sq, 6);   // <D, L D>
-    const double q =
-        qL + __shfl_sync(full, Sq, 4) - 2.0 * cfg.inv_eps * __shfl_sync(full, Sq, 2);  // <D, H D>
-    const double E = __longlong_as_double(static_cast<long long>(__shfl_sync(full, w, 16)));
-    const double g0in = __longlong_as_double(static_cast<long long>(__shfl_sync(full, w, 17)));
+    StepIn in;
+    in.E = __longlong_as_double(static_cast<long long>(__shfl_sync(full, w, 16)));
+    in.g0 = __longlong_as_double(static_cast<long long>(__shfl_sync(full, w, 17)));
     const unsigned long long ig = __shfl_sync(full, w, 18);
-    const int iter = int(static_cast<unsigned>(ig));
-    const int g0_set = int(static_cast<unsigned>(ig >> 32));
+    in.iter = int(static_cast<unsigned>(ig));
+    in.g0_set = int(static_cast<unsigned>(ig >> 32));
     const int err = int(__shfl_sync(full, w, 19));
-    const double g0 = g0_set ? g0in : g;
-    int status = 2;  // FW_PENDING
-    int done = 0;
-    if (err) {
-        status = -7;  // FW_ERR_TIMEOUT
-        done = 1;
-    } else if (nonfinite) {
-        status = -6;  // FW_ERR_NUMERIC
-        done = 1;
-    } else if (active == 0 || g <= 0.0) {
-        status = 0;
-        done = 1;
-    } else if (g <= (cfg.tol_mode ? cfg.gap_tol * g0 : cfg.gap_tol)) {
-        status = 0;
-        done = 1;
-    } else if (iter >= cfg.max_iters) {
-        status = 1;  // FW_NOT_CONVERGED
-        done = 1;
-    } else if (!isfinite(q)) {
-        status = -6;
-        done = 1;
-    }
-    double a = 1.0;
-    if (!done && q > 0.0) {
-        const double r = g / q;   // one division serves both rules
-        if (cfg.step_rule == 0) {
-            a = fmin(1.0, r);
-        } else {
-            // Armijo: largest 0.5^j with E(U) - E(U + a D) = a g - a^2 q / 2 >= 1e-6 a g,
-            // i.e. a <= 2 (1 - 1e-6) g / q
-            const double amax = 2.0 * (1.0 - 1e-6) * r;
-            for (int j = 0; j < 1100 && a > amax; ++j) a *= 0.5;
-        }
-    }
-    if (commit) {
-        if (lane == 0) st->g = Sq;
-        if (lane == 2) st->nD = Sq;
-        if (lane == 4) st->nW = Sq;
-        if (lane == 6) st->tLU = Sq;
-        if (lane == 8) st->active = int(Sq);
-        if (lane == 10) st->pLS = Sq;
-        if (lane == 0) {
-            st->g0 = g0;
-            st->g0_set = 1;
-            st->status = status;
-            st->done = done;
-            StepIn nx;
-            nx.E = E;
-            nx.g0 = g0;
-            nx.iter = iter;
-            nx.g0_set = 1;
-            if (!done) {
-                st->q = q;
-                st->alpha = a;
-                st->alpha_f = float(a);
-                nx.E = E - a * g + 0.5 * a * a * q;
-                nx.iter = iter + 1;
-            }
-            st->has_update = done ? 0 : 1;
-            st->E = nx.E;
-            st->iter = nx.iter;
-            st->in[c ^ 1] = nx;
-        }
-    }
-    *alpha = a;
-    return done;
+    const Decision d = decide(w, in, err, cfg);
+    if (commit) commit_decision(st, d, next_in(in, d), c ^ 1);
+    *alpha = d.a;
+    return d.done;
 }
 
 // k_finish and the persistent kernel's last block: one warp decides on bank

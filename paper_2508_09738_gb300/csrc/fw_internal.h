@@ -59,9 +59,40 @@ public:
     virtual size_t tab_smem(int lanes, int64_t n) const = 0;
 };
 
+// The resident kernel's launch of one problem (fw_resident.cuh).
+struct ResPlan {
+    int32_t group = 0;     // blocks that share the problem (0: the kernel does not apply)
+    int32_t cluster = 0;   // 1: they are one thread-block cluster, 0: a cooperative grid
+    int32_t layers = 0;    // 512-row layers of the fullest block
+    int32_t form = 0;      // kResShared, kResNarrow or kResWide
+    size_t smem = 0;       // dynamic shared memory of a block
+    int32_t direct = 0;    // rows walked in place (ResProb::direct)
+    int64_t slack = 0;     // entries added to each block's range of the slices
+    int64_t entries = 0;   // entries of the slices
+    size_t welem = 0;      // bytes of a weight
+};
+struct ResArgs;
+struct ResProb;
+class ResKern {
+public:
+    virtual ~ResKern() {}
+    // Whether (and how) the kernel takes this problem on the current device;
+    // maxrow: entries of the longest row.  share: layers a block should hold
+    // where other problems run beside this one (0: it has the device to itself).
+    virtual bool plan(const ProbDesc& pd, int maxrow, int64_t nnz_pad, int sms, int share,
+                      ResPlan& p) = 0;
+    // Fill the slices `prob` names.
+    virtual cudaError_t slice(const ResProb& prob, const ResPlan& p, cudaStream_t s) = 0;
+    // After the slices are built: most chunks of a block, from ResSlices::chunks.
+    virtual void sliced(ResPlan& p, int chunks) = 0;
+    virtual cudaError_t launch(const ResArgs& a, const ResPlan& p, cudaStream_t s) = 0;
+};
+// NULL when no resident kernel is compiled for K classes.
+ResKern* make_res(int weight_dtype, int K);
+
 // Non-template kernels (defined in fw_seg.cu).
 __global__ void k_validate(int64_t n, const int32_t* rp, const int32_t* col, const double* w,
-                           double* deg, int* err);
+                           double* deg, int* err, int* band);
 __global__ void k_state_init(ProbState* st, const double* part, int nb);
 __global__ void k_fid(int64_t n, const int32_t* labels, int8_t* fid);
 
@@ -86,6 +117,7 @@ struct HostGraph {
 struct ProbLayout {
     int64_t n = 0, nnz = 0, nnz_pad = 0, npad = 0;
     int32_t K = 0, tile_rows = 0, ntiles = 0, lanes = 1;
+    int32_t maxrow = 0;    // entries of the longest row
     // keep the 4-bit class array (ProbDesc::cls4): set by the two-kernel
     // single-problem path for K <= 16; the persistent kernels do not use it
     bool cls4 = false;

@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "fw_internal.h"
+#include "fw_resident.cuh"
 
 namespace fw {
 const char* last_error_text();
@@ -61,7 +62,10 @@ struct fw_seg {
     uint8_t* d_ch = nullptr;        // choice scratch of fw_seg_get_grad
     int32_t* d_labels = nullptr;
     double* d_opart = nullptr;
-    cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph = nullptr;   // NULL with a resident plan, and on streams without capture
+    std::unique_ptr<ResKern> res;      // solves run resident when res_plan.group > 0
+    ResPlan res_plan;
+    ResArgs res_args{};                // its launch parameters but the iteration count
     int last_refresh = 0;
     int launches = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -90,6 +94,9 @@ struct fw_seg {
         if (own_stream && stream) cudaStreamDestroy(stream);
     }
 };
+
+// Iterations of one resident launch (a few tens of ms at most).
+constexpr int kResIters = 4096;
 
 static fw_status launch_check(const char* what) {
     cudaError_t e = cudaGetLastError();
@@ -163,6 +170,41 @@ static void iteration(fw_seg* h) {
 // iteration but the last is taken inside the next pass A, so only the last
 // iteration ends with k_finish.
 static int graph_launches(int m) { return 2 * m + 1; }
+
+// Plan the resident kernel for the assembled problem and lay out its slices.
+// Without a plan, or without the memory for it, the solve runs the two-kernel
+// path.  The slices and the handle's other arrays stay within
+// fw_seg_footprint (create's temporaries are gone by now) plus 64 KB, less than
+// the granularity of the pool, so callers that admit by it need not know.
+static fw_status plan_resident(fw_seg* h) {
+    if (h->opts.class_table != FW_TABLE_AUTO) return FW_OK;   // the caller asks for a pass B form
+    h->res.reset(make_res(h->opts.weight_dtype, h->lay.K));
+    if (!h->res) return FW_OK;
+    int sms = 0;
+    FW_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    ResPlan p;
+    if (!h->res->plan(h->pd, h->lay.maxrow, h->lay.nnz_pad, sms, 0, p)) return FW_OK;
+    const ProbLayout& lay = h->lay;
+    const size_t te = h->ops->elem(), n = size_t(lay.n);
+    const size_t used = problem_bytes(lay, te, h->ops->welem(), h->pd.comb) + sizeof(ProbState) +
+                        te * size_t(lay.npad) * size_t(lay.K) + 5 * n + 8 * (n / kBlock + 1);
+    if (used + res_bytes(p) >
+        fw_seg_footprint(lay.n, lay.nnz, lay.K, h->opts.weight_dtype) + 65536)
+        return FW_OK;
+    char* m = nullptr;
+    if (h->alloc(&m, res_bytes(p)) != FW_OK) return FW_OK;
+    h->res_args = res_args(p, h->pd, h->st, m);
+    FW_CUDA(res_build(h->res.get(), h->res_args, p, h->stream));
+    h->res_plan = p;
+    return FW_OK;
+}
+
+// Up to `iters` iterations in one resident launch (it ends at the stop rule).
+static fw_status launch_resident(fw_seg* h, int iters) {
+    FW_CUDA(res_launch(h->res.get(), h->res_args, h->res_plan, iters, h->stream));
+    ++h->launches;
+    return FW_OK;
+}
 
 static fw_status build_graph(fw_seg* h) {
     if (h->graph) {
@@ -371,8 +413,8 @@ fw_status fw_seg_create(fw_seg** out, int64_t n, const int32_t* row_ptr, const i
             FW_CUDA(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
             h->own_stream = true;
         }
-        Upload up(h->stream);
-        FW_TRY(upload_inputs(g, up));
+        std::unique_ptr<Upload> up(new Upload(h->stream));
+        FW_TRY(upload_inputs(g, *up));
         if (upload_first) FW_TRY(plan_problem(g, o, h->lay));
         h->lay.cls4 = K <= 16;   // pass B gathers 4-bit classes (KMAX <= 16 forms)
         h->ops.reset(make_ops(o.weight_dtype, K));
@@ -394,9 +436,11 @@ fw_status fw_seg_create(fw_seg** out, int64_t n, const int32_t* row_ptr, const i
         FW_TRY(h->alloc(&h->d_ch, size_t(lay.n)));
         FW_TRY(h->alloc(&h->d_labels, 4 * size_t(lay.n)));
         FW_TRY(h->alloc(&h->d_opart, 8 * size_t((lay.n + kBlock - 1) / kBlock)));
-        FW_TRY(assemble_uploaded(h->ops.get(), up, lay, h->pd, h->st, h->stream));
+        FW_TRY(assemble_uploaded(h->ops.get(), *up, lay, h->pd, h->st, h->stream));
+        up.reset();   // its device copies go back to the pool
+        FW_TRY(plan_resident(h.get()));
         FW_TRY(read_state(h.get()));
-        if (build_graph(h.get()) != FW_OK) {
+        if (h->res_plan.group == 0 && build_graph(h.get()) != FW_OK) {
             // streams that cannot be captured (the legacy default stream) run
             // the same kernels as direct launches
             cudaGetLastError();
@@ -446,7 +490,13 @@ fw_status fw_seg_solve(fw_seg* h, fw_seg_stats* stats) {
     while (!h->h_state->done) {
         if (R > 0 && h->h_state->iter - h->last_refresh >= R) FW_TRY(refresh_lu(h));
         const int remaining = h->opts.max_iters - h->h_state->iter;
-        if (remaining >= m && h->graph) {
+        if (h->res_plan.group > 0) {
+            // the whole solve in one launch: its last evaluation meets the
+            // iteration cap.  With refreshes, as many iterations at a time as
+            // a graph holds.
+            const int it = R > 0 && remaining >= m ? m : std::min(remaining, kResIters) + 1;
+            FW_TRY(launch_resident(h, it));
+        } else if (remaining >= m && h->graph) {
             FW_CUDA(cudaGraphLaunch(h->graph, h->stream));
             h->launches += graph_launches(m);
         } else {
@@ -497,15 +547,22 @@ fw_status fw_seg_profile(fw_seg* h, int32_t iters, double* ms_a, double* ms_b, d
             cudaEventDestroy(b);
         }
     } guard{e0, e1};
-    // 1. the solve's own form: m fused iterations and one finish
+    // 1. the solve's own form: m fused iterations and one finish, or one
+    //    resident launch
     float t_ab = 0.f, t_a = 0.f, t_b = 0.f, t_f = 0.f;
+    fw_status res = FW_OK;
     FW_TRY(time_enqueued(h, graph, [&] {
+        if (h->res_plan.group > 0) {
+            res = launch_resident(h, m);
+            return;
+        }
         for (int i = 0; i < m; ++i) {
             h->ops->passA(h->pd, h->st, h->stream, i > 0 ? 1 : 0);
             h->ops->passB(h->pd, h->st, h->stream);
         }
         h->ops->finish(h->pd, h->st, h->stream);
     }, e0, e1, &t_ab));
+    FW_TRY(res);
     FW_TRY(read_state(h));
     if (h->h_state->done)
         return invalid("the stop rule held while profiling: reset and profile fewer iterations");

@@ -21,42 +21,46 @@ namespace fw {
 // Validation and degrees of the input CSR (one thread per row):
 //   columns strictly increasing and in range, no self loop, w finite and >= 0,
 //   w_ij == w_ji (binary search in row j), d_i = sum_j w_ij > 0 (Sec. 1).
-// err bits: 1 graph structure / weights, 2 asymmetric, 4 isolated node,
-// 8 (not an error) some |j - i| >= 2^15, so 16-bit column offsets cannot hold it.
+// err bits: 1 graph structure / weights, 2 asymmetric, 4 isolated node.
+// *band = max |j - i|, at most 2^15 - 1 when 16-bit column offsets can hold it.
 __global__ void k_validate(int64_t n, const int32_t* rp, const int32_t* col, const double* w,
-                           double* deg, int* err) {
+                           double* deg, int* err, int* band) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int e0 = rp[i], e1 = rp[i + 1];
-    double d = 0.0;
     int bad = 0, far = 0;
-    int prev = -1;
-    for (int e = e0; e < e1; ++e) {
-        const int j = col[e];
-        const double x = w[e];
-        if (j < 0 || j >= n || j == i || j <= prev || !(x >= 0.0) || isinf(x)) {
-            bad |= 1;
-            break;
-        }
-        prev = j;
-        d += x;
-        far |= (j - int(i) > 32767) | (int(i) - j > 32767);
-        int lo = rp[j], hi = rp[j + 1] - 1, pos = -1;
-        while (lo <= hi) {
-            const int mid = (lo + hi) >> 1;
-            const int cm = col[mid];
-            if (cm == i) {
-                pos = mid;
+    if (i < n) {
+        const int e0 = rp[i], e1 = rp[i + 1];
+        double d = 0.0;
+        int prev = -1;
+        for (int e = e0; e < e1; ++e) {
+            const int j = col[e];
+            const double x = w[e];
+            if (j < 0 || j >= n || j == i || j <= prev || !(x >= 0.0) || isinf(x)) {
+                bad |= 1;
                 break;
             }
-            if (cm < i) lo = mid + 1;
-            else hi = mid - 1;
+            prev = j;
+            d += x;
+            far = max(far, abs(j - int(i)));
+            int lo = rp[j], hi = rp[j + 1] - 1, pos = -1;
+            while (lo <= hi) {
+                const int mid = (lo + hi) >> 1;
+                const int cm = col[mid];
+                if (cm == i) {
+                    pos = mid;
+                    break;
+                }
+                if (cm < i) lo = mid + 1;
+                else hi = mid - 1;
+            }
+            if (pos < 0 || w[pos] != x) bad |= 2;
         }
-        if (pos < 0 || w[pos] != x) bad |= 2;
+        if (!bad && !(d > 0.0)) bad |= 4;
+        deg[i] = d;
     }
-    if (!bad && !(d > 0.0)) bad |= 4;
-    deg[i] = d;
-    if (bad | far) atomicOr(err, bad | (far ? 8 : 0));
+    if (bad) atomicOr(err, bad);
+    __syncwarp();
+    far = __reduce_max_sync(0xffffffffu, far);
+    if ((threadIdx.x & 31) == 0) atomicMax(band, far);
 }
 
 __global__ void __launch_bounds__(kBlock) k_state_init(ProbState* st, const double* part, int nb) {
@@ -204,6 +208,25 @@ Ops* make_ops(int weight_dtype, int K) {
     }
 }
 
+ResKern* make_res_f32_lo(int K);
+ResKern* make_res_f32_hi(int K);
+ResKern* make_res_f32_top(int K);
+ResKern* make_res_bf16_lo(int K);
+ResKern* make_res_bf16_hi(int K);
+ResKern* make_res_bf16_top(int K);
+ResKern* make_res_f64(int K);
+
+ResKern* make_res(int weight_dtype, int K) {
+    switch (weight_dtype) {
+        case FW_WEIGHTS_F32:
+            return K <= 6 ? make_res_f32_lo(K) : K <= 10 ? make_res_f32_hi(K) : make_res_f32_top(K);
+        case FW_WEIGHTS_BF16:
+            return K <= 6 ? make_res_bf16_lo(K) : K <= 10 ? make_res_bf16_hi(K) : make_res_bf16_top(K);
+        case FW_WEIGHTS_F64: return make_res_f64(K);
+        default: return nullptr;
+    }
+}
+
 int tile_rows_for(int64_t n) {
     const int64_t sub = (n + kBlock - 1) / kBlock;               // 256-row sub-tiles
     const int64_t per = (sub + kTilesTarget - 1) / kTilesTarget;  // sub-tiles per tile
@@ -266,22 +289,24 @@ fw_status plan_problem(const HostGraph& g, const fw_seg_opts& o, ProbLayout& lay
     // themselves are formed on the device): a negative row length sets the
     // sign bit of `neg`.  Large inputs are split over a few host threads.
     struct Part {
-        int64_t acc = 0, neg = 0;
+        int64_t acc = 0, neg = 0, longest = 0;
         int bad = 0;
     };
     auto scan_part = [&g](int64_t i0, int64_t i1, Part& p) {
         const int32_t* __restrict__ rp = g.rp;
         const int32_t* __restrict__ lab = g.labels;
-        int64_t acc = 0, neg = 0;
+        int64_t acc = 0, neg = 0, longest = 0;
         int bad = 0;
         for (int64_t i = i0; i < i1; ++i) {
             const int64_t d = int64_t(rp[i + 1]) - int64_t(rp[i]);
             neg |= d;
+            longest = std::max(longest, d);
             acc += (d + (kPadW - 1)) & ~int64_t(kPadW - 1);
             bad |= int(lab[i] < -1) | int(lab[i] >= g.K);
         }
         p.acc = acc;
         p.neg = neg;
+        p.longest = longest;
         p.bad = bad;
     };
     const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
@@ -304,10 +329,11 @@ fw_status plan_problem(const HostGraph& g, const fw_seg_opts& o, ProbLayout& lay
         parts.assign(1, Part());
         scan_part(0, n, parts[0]);
     }
-    int64_t acc = 0, neg = 0;
+    int64_t acc = 0, neg = 0, longest = 0;
     int bad = 0;
     for (const Part& p : parts) {
         acc += p.acc;
+        longest = std::max(longest, p.longest);
         neg |= p.neg;
         bad |= p.bad;
     }
@@ -323,6 +349,7 @@ fw_status plan_problem(const HostGraph& g, const fw_seg_opts& o, ProbLayout& lay
     lay.n = n;
     lay.nnz = g.rp[n];
     lay.nnz_pad = acc;
+    lay.maxrow = int32_t(longest);
     if (lay.nnz > 0 && (!g.col || !g.w)) return invalid("col and w must not be NULL");
     lay.npad = round_up(n, 32);
     lay.K = g.K;
@@ -551,7 +578,7 @@ fw_status assemble_uploaded(Ops* ops, Upload& up, const ProbLayout& lay, ProbDes
     double* d_deg = nullptr;
     int* d_err = nullptr;
     FW_TRYS(t.get(&d_deg, 8 * size_t(n)));
-    FW_TRYS(t.get(&d_err, sizeof(int)));
+    FW_TRYS(t.get(&d_err, 2 * sizeof(int)));   // error bits, bandwidth
     {   // padded row offsets into pd.rp
         const int nb = int((n + kScanRows - 1) / kScanRows);
         int32_t* d_bsum = nullptr;
@@ -565,13 +592,14 @@ fw_status assemble_uploaded(Ops* ops, Upload& up, const ProbLayout& lay, ProbDes
     const size_t blk = te * size_t(lay.npad) * size_t(lay.K);
     FW_CUDA(cudaMemsetAsync(pd.U, 0, blk, s));
     FW_CUDA(cudaMemsetAsync(pd.LS, 0, blk, s));
-    FW_CUDA(cudaMemsetAsync(d_err, 0, sizeof(int), s));
+    FW_CUDA(cudaMemsetAsync(d_err, 0, 2 * sizeof(int), s));
     const unsigned gr = unsigned((n + kBlock - 1) / kBlock);
-    k_validate<<<gr, kBlock, 0, s>>>(n, d_rp, d_col, d_w, d_deg, d_err);
+    k_validate<<<gr, kBlock, 0, s>>>(n, d_rp, d_col, d_w, d_deg, d_err, d_err + 1);
     FW_TRYS(launched("validate kernel"));
-    int err = 0;
-    FW_CUDA(cudaMemcpyAsync(&err, d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    int checked[2] = {0, 0};
+    FW_CUDA(cudaMemcpyAsync(checked, d_err, sizeof(checked), cudaMemcpyDeviceToHost, s));
     FW_CUDA(cudaStreamSynchronize(s));
+    const int err = checked[0];
     if (err & 3) {
         set_error(err & 1 ? "graph: column out of range / not increasing / self loop / bad weight"
                           : "graph: W is not symmetric");
@@ -583,7 +611,8 @@ fw_status assemble_uploaded(Ops* ops, Upload& up, const ProbLayout& lay, ProbDes
     }
     // banded graphs (pixel grids, meshes) keep 16-bit column offsets: the
     // same entries in half the column bytes of every sparse pass
-    pd.col16 = (lay.allow16 && !(err & 8)) ? 1 : 0;
+    pd.band = checked[1];
+    pd.col16 = (lay.allow16 && pd.band < 1 << 15) ? 1 : 0;
     FW_TRYS(choose_tab(ops, lay, pd));
     if (!pd.comb) k_inv_sqrt<<<gr, kBlock, 0, s>>>(n, d_deg);
     ops->build(n, d_rp, d_col, d_w, d_deg, pd.rp, const_cast<int32_t*>(pd.col),
