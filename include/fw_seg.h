@@ -262,7 +262,9 @@ void fw_seg_destroy(fw_seg *h);
  *
  * All problems of a batch live in one contiguous device pool (each at its own
  * offsets) and iterate together, from a captured CUDA graph, in one of two
- * schedules (FW_SCHED_*): per-item launches, where each iteration is one
+ * schedules (FW_SCHED_*): per-item launches, where the problems that the
+ * resident kernel of fw_seg_solve takes run in one such launch each, beside
+ * each other, and each iteration of the rest is one
  * launch of pass A over the row tiles of every live problem and one of pass B
  * (the kernel boundaries are the barriers); or a cooperative persistent
  * kernel: phase A, grid barrier, phase B, grid barrier, per iteration.  Each
@@ -377,7 +379,9 @@ void fw_batch_destroy(fw_batch *b);
  * the only resident below that size -- or else one batched epoch over the
  * residents below that size (a large one waits until it is the oldest):
  * per-item launches (the default) or the persistent kernel
- * (FW_SCHED_STATIC / FW_SCHED_DYNAMIC).
+ * (FW_SCHED_STATIC / FW_SCHED_DYNAMIC).  Under the default schedule requests
+ * that the resident kernel takes need no shared epochs: each keeps two
+ * launches of four epochs' iterations in flight on a stream of its own.
  * Lone-request epochs run from a captured graph, two kept in flight ahead of
  * the worker thread.
  * Requests that meet their stop rule are harvested

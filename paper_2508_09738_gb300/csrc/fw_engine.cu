@@ -26,6 +26,7 @@
 
 #include "fw_batch.cuh"
 #include "fw_internal.h"
+#include "fw_resident.cuh"
 
 namespace fw {
 
@@ -112,7 +113,16 @@ struct Slot {
     ProbDesc pd{};
     fw_seg_opts opts{};
     size_t off = 0, bytes = 0;
+    // the resident kernel takes the problem when res.group > 0
+    ResPlan res;
+    ResArgs rargs{};
+    ResKern* rk = nullptr;
+    size_t roff = SIZE_MAX, rbytes = 0;   // its arrays in the pool,
+    void* rmem = nullptr;                 // or in the library's pool
+    int rhead = 0, rqueued = 0;           // serving: launches in flight (ring entries)
 };
+
+constexpr int kResStreams = 32;   // streams the resident launches of a batch spread over
 
 class Engine {
 public:
@@ -156,6 +166,19 @@ public:
     ProbState* h_ring = nullptr;                 // pinned [2]
     cudaEvent_t ring_ev[2] = {nullptr, nullptr};
     int ring_head = 0, ring_queued = 0;
+    // Resident problems run beside each other, each launch on its own few SMs:
+    // slot s on stream s mod kResStreams.  30 k-NN problems (1,000 to 60,000
+    // points, 200 iterations, BF16): 14.3 ms a batch with two launches per
+    // iteration over all tiles, 10.1 with one resident launch each; a burst of
+    // 12 served requests 21.6 -> 16.2 ms.
+    std::map<int, std::unique_ptr<ResKern>> reskern;   // per class count
+    cudaStream_t rstream[kResStreams] = {};
+    cudaEvent_t rfork = nullptr, rjoin[kResStreams] = {};
+    std::vector<int> h_res;                      // live slots with a plan
+    ProbState* h_rring = nullptr;                // pinned [slots][2] (serving)
+    std::vector<cudaEvent_t> rring_ev;           // [slots][2]
+    bool res_outside = false;                    // slices may come from the library's pool
+    int res_share = 0;                           // ResKern::plan
     long long budget = 0;
     cudaGraphExec_t graph = nullptr;
     int graph_iters = -1;
@@ -166,8 +189,19 @@ public:
     ~Engine() {
         if (stream) cudaStreamSynchronize(stream);
         if (side) cudaStreamSynchronize(side);
+        for (cudaStream_t r : rstream)
+            if (r) cudaStreamSynchronize(r);
         if (graph) cudaGraphExecDestroy(graph);
         if (lone_graph) cudaGraphExecDestroy(lone_graph);
+        for (Slot& sl : slots)
+            if (sl.rmem) cudaFreeAsync(sl.rmem, side);
+        for (cudaStream_t r : rstream)
+            if (r) cudaStreamDestroy(r);
+        if (rfork) cudaEventDestroy(rfork);
+        for (cudaEvent_t ev : rjoin)
+            if (ev) cudaEventDestroy(ev);
+        for (cudaEvent_t ev : rring_ev) cudaEventDestroy(ev);
+        if (h_rring) cudaFreeHost(h_rring);
         for (cudaEvent_t ev : ring_ev)
             if (ev) cudaEventDestroy(ev);
         if (h_ring) cudaFreeHost(h_ring);
@@ -270,9 +304,15 @@ public:
         for (int s = 0; s < nslots(); ++s) {
             Slot& sl = slots[size_t(s)];
             if (!sl.used) continue;
-            sl.pd.lanes = L > 0 ? L : sl.lay.lanes;
+            const int lanes = L > 0 ? L : sl.lay.lanes;
+            if (lanes == sl.pd.lanes) continue;
+            sl.pd.lanes = lanes;
             FW_CUDA(cudaMemcpyAsync(d_desc + s, &sl.pd, sizeof(ProbDesc), cudaMemcpyHostToDevice,
                                     stream));
+            if (sl.res.group > 0) {   // the slices hold the sums' order
+                drop_res(sl);
+                FW_TRY(plan_res(s));
+            }
         }
         FW_CUDA(cudaStreamSynchronize(stream));
         invalidate_graph();
@@ -343,7 +383,91 @@ public:
         sl.used = true;
         work_dirty = true;
         *out = s;
+        if (plain_path && schedule == FW_SCHED_ITEMS) {
+            // small requests alone on their SMs, larger ones two layers a
+            // block so that several fit beside each other
+            res_share = lay.ntiles <= kResTilesPerLayer * kResMaxCluster ? 1 : 2;
+            if (lay.n >= shared_max_rows) res_share = 0;
+            rc = plan_res(s);
+            if (rc != FW_OK) remove(s);
+        }
+        return rc;
+    }
+
+    // Plan slot s for the resident kernel and lay out its slices, in the pool
+    // (keeping a quarter of it free for admissions) or, for a batch, in the
+    // library's pool.  Without room the slot runs as items.
+    fw_status plan_res(int s) {
+        Slot& sl = slots[size_t(s)];
+        auto it = reskern.find(sl.lay.K);
+        if (it == reskern.end())
+            it = reskern.emplace(sl.lay.K, std::unique_ptr<ResKern>(make_res(wd, sl.lay.K))).first;
+        ResKern* k = it->second.get();
+        ResPlan p;
+        if (!k || !k->plan(sl.pd, sl.lay.maxrow, sl.lay.nnz_pad, sms, res_share, p)) return FW_OK;
+        const size_t need = res_bytes(p);
+        char* m = nullptr;
+        size_t off = SIZE_MAX;
+        void* outside = nullptr;
+        if (res_outside) {
+            if (pool_alloc(&outside, need, side) != FW_OK) return FW_OK;
+            m = static_cast<char*>(outside);
+        } else {
+            if (ra.cap() - ra.used() < need + ra.cap() / 4) return FW_OK;
+            off = ra.alloc(need);
+            if (off == SIZE_MAX) return FW_OK;
+            m = pool + off;
+        }
+        sl.rargs = res_args(p, sl.pd, d_state + s, m);
+        sl.roff = off;
+        sl.rmem = outside;
+        sl.rbytes = need;
+        sl.rk = k;
+        FW_CUDA(res_build(k, sl.rargs, p, side));
+        sl.res = p;
+        sl.rhead = sl.rqueued = 0;
+        if (!rfork) {
+            FW_CUDA(cudaEventCreateWithFlags(&rfork, cudaEventDisableTiming));
+            for (int i = 0; i < kResStreams; ++i) {
+                FW_CUDA(cudaStreamCreateWithFlags(&rstream[i], cudaStreamNonBlocking));
+                FW_CUDA(cudaEventCreateWithFlags(&rjoin[i], cudaEventDisableTiming));
+            }
+        }
         return FW_OK;
+    }
+    // Give the slot's resident arrays back (none of its launches in flight).
+    void drop_res(Slot& sl) {
+        if (sl.roff != SIZE_MAX) ra.release(sl.roff, sl.rbytes);
+        if (sl.rmem) cudaFreeAsync(sl.rmem, side);
+        sl.roff = SIZE_MAX;
+        sl.rmem = nullptr;
+        sl.res = ResPlan();
+        sl.rk = nullptr;
+    }
+    // The streams resident slots have launches on, forked from `stream` and
+    // joined back into it around `iters` iterations of every slot of h_res.
+    cudaError_t enqueue_res(int iters) {
+        if (h_res.empty()) return cudaSuccess;
+        cudaError_t e = cudaEventRecord(rfork, stream);
+        bool used[kResStreams] = {};
+        // most work first: the device fills with the small ones beside it
+        std::vector<int> order = h_res;
+        std::stable_sort(order.begin(), order.end(), [this](int x, int y) {
+            return slots[size_t(x)].lay.n > slots[size_t(y)].lay.n;
+        });
+        for (size_t i = 0; i < order.size() && e == cudaSuccess; ++i) {
+            const int q = int(i) % kResStreams;
+            if (!used[q]) e = cudaStreamWaitEvent(rstream[q], rfork, 0);
+            used[q] = true;
+            const Slot& sl = slots[size_t(order[i])];
+            if (e == cudaSuccess) e = res_launch(sl.rk, sl.rargs, sl.res, iters, rstream[q]);
+        }
+        for (int q = 0; q < kResStreams && e == cudaSuccess; ++q) {
+            if (!used[q]) continue;
+            e = cudaEventRecord(rjoin[q], rstream[q]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, rjoin[q], 0);
+        }
+        return e;
     }
 
     void remove(int s) {
@@ -355,6 +479,8 @@ public:
             lone_graph = nullptr;
             lone_slot = -1;
         }
+        if (sl.rqueued) cudaStreamSynchronize(rstream[s % kResStreams]);
+        drop_res(sl);
         ra.release(sl.off, sl.bytes);
         sl = Slot();
         work_dirty = true;
@@ -371,23 +497,28 @@ public:
     // Work list of the live problems (used, not done, below shared_max_rows).
     int build_work() {
         std::vector<int2> w;
-        std::vector<int> live;
+        std::vector<int> live, res;
         bool two = false;
         for (int s = 0; s < nslots(); ++s) {
             if (!slots[size_t(s)].used || h_state[s].done) continue;
             if (slots[size_t(s)].lay.n >= shared_max_rows) continue;
+            if (schedule == FW_SCHED_ITEMS && slots[size_t(s)].res.group > 0) {
+                res.push_back(s);
+                continue;
+            }
             live.push_back(s);
             two = two || slots[size_t(s)].lay.tile_rows > kBlock;
             for (int t = 0; t < slots[size_t(s)].lay.ntiles; ++t) w.push_back(make_int2(s, t));
         }
-        if (w.size() != h_work.size() || live != h_live ||
+        if (w.size() != h_work.size() || live != h_live || res != h_res ||
             !std::equal(w.begin(), w.end(), h_work.begin(),
                         [](const int2& x, const int2& y) { return x.x == y.x && x.y == y.y; }))
             work_dirty = true;
         h_work.swap(w);
         h_live.swap(live);
+        h_res.swap(res);
         two_stage = two;
-        return int(h_live.size());
+        return int(h_live.size() + h_res.size());
     }
 
     fw_status ensure_work_cap(size_t n) {
@@ -422,10 +553,12 @@ public:
         if (nlive == 0) return FW_OK;
         if (work_dirty) {
             FW_TRY(ensure_work_cap(h_work.size()));
-            FW_CUDA(cudaMemcpyAsync(d_work, h_work.data(), sizeof(int2) * h_work.size(),
-                                    cudaMemcpyHostToDevice, stream));
-            FW_CUDA(cudaMemcpyAsync(d_live, h_live.data(), sizeof(int) * h_live.size(),
-                                    cudaMemcpyHostToDevice, stream));
+            if (!h_work.empty()) {
+                FW_CUDA(cudaMemcpyAsync(d_work, h_work.data(), sizeof(int2) * h_work.size(),
+                                        cudaMemcpyHostToDevice, stream));
+                FW_CUDA(cudaMemcpyAsync(d_live, h_live.data(), sizeof(int) * h_live.size(),
+                                        cudaMemcpyHostToDevice, stream));
+            }
             invalidate_graph();
             work_dirty = false;
         }
@@ -433,13 +566,16 @@ public:
         const ItemArgs ia{d_desc, d_state, d_work, d_live};
         const bool items = schedule == FW_SCHED_ITEMS;
         // one launch's work: the barrier record cleared, then the persistent
-        // kernel or the per-item launches
+        // kernel, or the resident launches and the per-item launches of the rest
         auto enqueue = [&]() -> cudaError_t {
             cudaError_t e = cudaMemsetAsync(d_bar, 0, sizeof(GridBar), stream);
             if (e != cudaSuccess) return e;
-            if (items)
-                return bk->launch_items(ia, int(h_work.size()), nlive, iters, two_stage, stream);
-            return bk->launch(a, grid, stream);
+            if (!items) return bk->launch(a, grid, stream);
+            e = enqueue_res(iters);
+            if (e == cudaSuccess && !h_work.empty())
+                e = bk->launch_items(ia, int(h_work.size()), int(h_live.size()), iters, two_stage,
+                                     stream);
+            return e;
         };
         bool from_graph = false;
         if (use_graph != FW_GRAPH_OFF) {
@@ -502,9 +638,18 @@ public:
         return cnt == 1 ? live : -1;
     }
 
-    // Wait for queued lone epochs; h_state then holds the device state.
+    // Wait for queued lone and resident launches; h_state then holds the
+    // device state.
     fw_status drain_lone() {
-        if (ring_queued == 0) return FW_OK;
+        bool any = ring_queued > 0;
+        for (int s = 0; s < nslots(); ++s) {
+            Slot& sl = slots[size_t(s)];
+            if (sl.rqueued == 0) continue;
+            FW_CUDA(cudaStreamSynchronize(rstream[s % kResStreams]));
+            sl.rqueued = sl.rhead = 0;
+            any = true;
+        }
+        if (!any) return FW_OK;
         ring_queued = 0;
         FW_CUDA(cudaStreamSynchronize(stream));
         FW_CUDA(cudaMemcpy(h_state, d_state, sizeof(ProbState) * slots.size(),
@@ -512,10 +657,56 @@ public:
         return FW_OK;
     }
 
+    // Serving: keep two launches of `iters` iterations in flight for each of
+    // these resident slots, each on the slot's stream, the state copied into
+    // the slot's pinned ring entry after each, so no problem waits for
+    // another or for the host.
+    fw_status res_queue(const std::vector<int>& set, int iters) {
+        if (ring_queued > 0) FW_TRY(drain_lone());
+        if (!h_rring) {
+            FW_CUDA(cudaMallocHost(&h_rring, 2 * slots.size() * sizeof(ProbState)));
+            for (size_t i = 0; i < 2 * slots.size(); ++i) {
+                cudaEvent_t ev = nullptr;
+                FW_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+                rring_ev.push_back(ev);
+            }
+        }
+        for (int round = 0; round < 2; ++round)
+            for (int s : set) {
+                Slot& sl = slots[size_t(s)];
+                if (sl.rqueued > round) continue;
+                const size_t i = 2 * size_t(s) + size_t((sl.rhead + sl.rqueued) & 1);
+                const cudaStream_t q = rstream[s % kResStreams];
+                FW_CUDA(res_launch(sl.rk, sl.rargs, sl.res, iters, q));
+                FW_CUDA(cudaMemcpyAsync(h_rring + i, d_state + s, sizeof(ProbState),
+                                        cudaMemcpyDeviceToHost, q));
+                FW_CUDA(cudaEventRecord(rring_ev[i], q));
+                ++sl.rqueued;
+            }
+        return FW_OK;
+    }
+    // The states after the oldest launch of each (the newer ones keep running).
+    fw_status res_collect(const std::vector<int>& set) {
+        for (int s : set) {
+            Slot& sl = slots[size_t(s)];
+            const size_t i = 2 * size_t(s) + size_t(sl.rhead);
+            FW_CUDA(cudaEventSynchronize(rring_ev[i]));
+            h_state[s] = h_rring[i];
+            sl.rhead ^= 1;
+            --sl.rqueued;
+        }
+        return FW_OK;
+    }
+
     // Queue lone epochs of `iters` iterations of slot s until two are in
     // flight.  false: the stream cannot be captured (nothing queued).
     fw_status lone_queue(int s, int iters, bool* ok) {
         *ok = false;
+        for (const Slot& sl : slots)
+            if (sl.rqueued > 0) {
+                FW_TRY(drain_lone());
+                break;
+            }
         if (!h_ring) {
             FW_CUDA(cudaMallocHost(&h_ring, 2 * sizeof(ProbState)));
             for (cudaEvent_t& ev : ring_ev)
@@ -704,7 +895,7 @@ static std::string tune_signature(const fw_batch* b) {
     cudaGetDevice(&dev);
     cudaGetDeviceProperties(&p, dev);
     char buf[512];
-    std::snprintf(buf, sizeof(buf), "v2|%s|wd%d|k%d|P%d|rows%lld|nnz%lld|tiles%lld|want%d%d%d%d",
+    std::snprintf(buf, sizeof(buf), "v3|%s|wd%d|k%d|P%d|rows%lld|nnz%lld|tiles%lld|want%d%d%d%d",
                   p.name, b->eng.wd, b->eng.kmax, b->P, (long long)rows, (long long)nnz,
                   (long long)tiles, b->bo.blocks_per_sm, b->bo.schedule, b->bo.lanes_per_row,
                   b->bo.iters_per_launch);
@@ -832,6 +1023,22 @@ static fw_status batch_tune(fw_batch* b) {
     c.sched = (o.schedule == FW_SCHED_STATIC || o.schedule == FW_SCHED_ITEMS) ? o.schedule
                                                                                : FW_SCHED_DYNAMIC;
     c.bps = o.blocks_per_sm > 0 ? std::min(o.blocks_per_sm, e.occ) : e.occ;
+    // When the resident kernel takes every problem nothing is left to time: it
+    // needs none of the dimensions, and the few iterations a candidate gets
+    // would count its start and not its iterations.
+    bool resident = o.schedule == FW_SCHED_AUTO || o.schedule == FW_SCHED_ITEMS;
+    for (const Slot& s : e.slots) resident = resident && s.res.group > 0;
+    if (resident) {
+        c.sched = FW_SCHED_ITEMS;
+        e.use_graph = keep_graph;
+        FW_TRY(apply_choice(b, c));
+        FW_TRY(batch_reset(b));
+        tune_store(b, sig, c);
+        b->tuned = 1;
+        b->tune_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0)
+                         .count();
+        return FW_OK;
+    }
     const int it = 4;
     float best = 1e30f, ms = 0.f;
     auto consider = [&](const TuneChoice& t, int iters, int per) -> fw_status {
@@ -975,6 +1182,16 @@ fw_status fw_batch_create(fw_batch** out, int32_t P, const fw_graph* graphs,
             const HostGraph hg{g.n, g.row_ptr_host, g.col_host, g.w_host, g.K, g.labels_host};
             int slot = -1;
             FW_TRY(e.add(hg, o, lays[size_t(p)], &slot));
+        }
+        if (b->bo.schedule == FW_SCHED_AUTO || b->bo.schedule == FW_SCHED_ITEMS) {
+            // as many layers a block as it takes to have every problem on the
+            // device at once, or as its registers hold
+            int64_t layers = 0;
+            for (const ProbLayout& l : lays)
+                layers += (l.ntiles + kResTilesPerLayer - 1) / kResTilesPerLayer;
+            e.res_share = int(std::min<int64_t>((layers + e.sms - 1) / e.sms, 4));
+            e.res_outside = true;
+            for (int p = 0; p < P; ++p) FW_TRY(e.plan_res(p));
         }
         b->ipl = std::max(0, b->bo.iters_per_launch);
         if (b->bo.blocks_per_sm <= 0 || b->bo.schedule == FW_SCHED_AUTO ||
@@ -1224,10 +1441,29 @@ void fw_srv::loop() {
             if (oldest >= 0 && e.slots[size_t(oldest)].lay.n >= kAloneRows) lone = oldest;
             else if (nsmall == 1) lone = small;
         }
+        // Requests the resident kernel takes run beside each other, without
+        // shared epochs: two launches of each are kept in flight.  They are
+        // longer than an epoch, since none of them holds up another.
+        std::vector<int> res;
+        for (int q = 0; q < e.nslots(); ++q) {
+            if (!e.slots[size_t(q)].used || e.h_state[q].done) continue;
+            if (lone >= 0 ? q != lone : e.slots[size_t(q)].lay.n >= kAloneRows) continue;
+            if (e.slots[size_t(q)].res.group == 0) {
+                res.clear();   // this one needs the shared epochs
+                break;
+            }
+            res.push_back(q);
+        }
         bool piped = false;
-        fw_status rc = lone >= 0 ? e.lone_queue(lone, iters, &piped) : FW_OK;
-        if (rc == FW_OK && piped) nlive = 1;
-        else if (rc == FW_OK) rc = e.launch_epoch(iters, &nlive);
+        fw_status rc = FW_OK;
+        if (!res.empty()) {
+            rc = e.res_queue(res, 4 * iters);
+            nlive = int(res.size());
+        } else {
+            rc = lone >= 0 ? e.lone_queue(lone, iters, &piped) : FW_OK;
+            if (rc == FW_OK && piped) nlive = 1;
+            else if (rc == FW_OK) rc = e.launch_epoch(iters, &nlive);
+        }
         // ... and admit queued requests (FIFO) while it runs: upload and
         // assembly go to the side stream, the pool range is taken in order
         for (;;) {
@@ -1261,7 +1497,7 @@ void fw_srv::loop() {
             }
         }
         if (rc == FW_OK && nlive > 0) {
-            rc = piped ? e.lone_collect() : e.collect();
+            rc = !res.empty() ? e.res_collect(res) : piped ? e.lone_collect() : e.collect();
             std::lock_guard<std::mutex> lk(mu);
             info.epochs++;
             for (int s = 0; s < e.nslots(); ++s)
