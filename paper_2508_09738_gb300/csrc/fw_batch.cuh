@@ -160,20 +160,22 @@ struct ItemArgs {
 };
 
 // Warp 0 copies the item's descriptor (8-byte words) into shared memory.
-__device__ __forceinline__ int2 item_desc(const ItemArgs& a, ProbDesc* s_pd) {
+__device__ __forceinline__ void item_desc(const ItemArgs& a, const int2& wk, ProbDesc* s_pd) {
     static_assert(sizeof(ProbDesc) % 8 == 0 && sizeof(ProbDesc) / 8 <= 32, "descriptor words");
-    const int2 wk = a.work[blockIdx.x];
     if (threadIdx.x < sizeof(ProbDesc) / 8)
         reinterpret_cast<unsigned long long*>(s_pd)[threadIdx.x] =
             reinterpret_cast<const unsigned long long*>(a.desc + wk.x)[threadIdx.x];
     __syncthreads();
-    return wk;
 }
 
 template <typename T, int KMAX>
-__global__ void __launch_bounds__(kBlock, passA_min_blocks<T, KMAX>()) k_itemA(ItemArgs a, int fin) {
+__global__ void __launch_bounds__(kBlock, passA_min_blocks<T, KMAX>()) k_itemA(ItemArgs a, int nwork, int fin) {
     __shared__ __align__(16) ProbDesc s_pd;
-    const int2 wk = item_desc(a, &s_pd);
+    // a fused launch has one block more per live problem (see passA_step)
+    const bool item = int(blockIdx.x) < nwork;
+    int2 wk = item ? a.work[blockIdx.x] : make_int2(a.live[int(blockIdx.x) - nwork], 0);
+    item_desc(a, wk, &s_pd);
+    if (!item) wk.y = s_pd.ntiles;
     extern __shared__ __align__(128) unsigned char smraw[];
     passA_step<T, KMAX, false>(s_pd, a.state + wk.x, fin, reinterpret_cast<T*>(smraw), wk.y);
 }
@@ -190,7 +192,8 @@ constexpr int itemB_min_blocks() {
 template <typename T, typename WT, int KMAX>
 __global__ void __launch_bounds__(kBlock, itemB_min_blocks<T, KMAX>()) k_itemB(ItemArgs a) {
     __shared__ __align__(16) ProbDesc s_pd;
-    const int2 wk = item_desc(a, &s_pd);
+    const int2 wk = a.work[blockIdx.x];
+    item_desc(a, wk, &s_pd);
     ProbState* st = a.state + wk.x;
     bool done;
     unsigned long long* accb = passB_bank(s_pd, st, done, wk.y);
@@ -258,7 +261,8 @@ public:
     cudaError_t launch_items(const ItemArgs& a, int nwork, int nlive, int iters, bool two_stage,
                              cudaStream_t s) override {
         for (int i = 0; i < iters; ++i) {
-            k_itemA<T, KMAX><<<nwork, kBlock, smem_itemA(two_stage), s>>>(a, i > 0 ? 1 : 0);
+            const int fin = i > 0 ? 1 : 0;
+            k_itemA<T, KMAX><<<nwork + fin * nlive, kBlock, smem_itemA(two_stage), s>>>(a, nwork, fin);
             k_itemB<T, WT, KMAX><<<nwork, kBlock, smem_itemB(), s>>>(a);
         }
         k_itemFinish<<<nlive, 32, 0, s>>>(a);

@@ -268,11 +268,43 @@ __device__ __forceinline__ bool fx_split(double v, unsigned long long& lo, unsig
     hi = static_cast<unsigned long long>(__double2ll_rz(fl));
     return true;
 }
-__device__ __forceinline__ void fx_add(unsigned long long* slot, unsigned long long* flag,
-                                       double v) {
+// Q64.64 of a tile total in the iterate type, the value fx_split gives for
+// double(v).  An FP32 total is shifted into place with integer instructions;
+// small negative ones (whose 1 - frac rounds in FP64) and large ones take
+// fx_split itself.
+__device__ __forceinline__ bool fx_total_split(double v, unsigned long long& lo,
+                                               unsigned long long& hi) {
+    return fx_split(v, lo, hi);
+}
+__device__ __forceinline__ bool fx_total_split(float v, unsigned long long& lo,
+                                               unsigned long long& hi) {
+    const uint32_t b = __float_as_uint(v);
+    const int ex = int((b >> 23) & 0xff);
+    const bool neg = (b >> 31) != 0;
+    // |v| < 2^40, and |v| >= 2^-29 when negative (then 1 - frac is exact)
+    if (ex >= 127 + 40 || (neg && ex < 127 - 29 && (b << 1) != 0u)) return fx_split(double(v), lo, hi);
+    const unsigned long long m = ex ? ((b & 0x7fffffu) | 0x800000u) : (b & 0x7fffffu);
+    const int sh = (ex ? ex : 1) - 150 + 64;   // v = m 2^(sh - 64)
+    if (sh >= 0) {
+        lo = sh < 64 ? m << sh : 0ull;
+        hi = sh >= 64 ? m << (sh - 64) : (sh > 40 ? m >> (64 - sh) : 0ull);
+    } else {
+        lo = sh > -64 ? m >> -sh : 0ull;
+        hi = 0ull;
+    }
+    if (neg) {
+        lo = ~lo + 1ull;
+        hi = ~hi + (lo == 0ull ? 1ull : 0ull);
+    }
+    return true;
+}
+
+// Add a tile total to the accumulator slot[].
+template <typename T>
+__device__ __forceinline__ void fx_add(unsigned long long* slot, unsigned long long* flag, T v) {
     static_assert(kTilesTarget < 2048, "fixed-point totals assume < 2^11 tiles");
     unsigned long long lo, hi;
-    if (!fx_split(v, lo, hi)) {
+    if (!fx_total_split(v, lo, hi)) {
         atomicOr(flag, 1ull);
         return;
     }
@@ -281,6 +313,12 @@ __device__ __forceinline__ void fx_add(unsigned long long* slot, unsigned long l
     atomicAdd(&slot[1], hi + carry);
 }
 
+// (lo, hi) += (l2, h2) in 128 bits.
+__device__ __forceinline__ void add128(unsigned long long& lo, unsigned long long& hi,
+                                       unsigned long long l2, unsigned long long h2) {
+    lo += l2;
+    hi += h2 + (lo < l2 ? 1ull : 0ull);
+}
 __device__ __forceinline__ unsigned long long* acc_slot(unsigned long long* acc, int copy, int q) {
     return acc + (copy * kNumR + q) * kAccLine;
 }
@@ -300,6 +338,33 @@ __device__ __forceinline__ double fx_total(const unsigned long long* acc, int q)
     return double(static_cast<long long>(hi)) + ldexp(double(lo), -64);
 }
 
+// Butterfly sums of six values over a warp (partners 16, 8, 4, 2, 1): at each of the first three steps half of
+// the lanes go on with one value and half with another, so 8 shuffles do the
+// work of 30 and every sum has the same bits.  Lane 0 returns x[0], 16 x[1],
+// 8 x[2], 24 x[3], 4 x[4], 20 x[5].
+template <typename T>
+__device__ __forceinline__ T warp_sum6(const T (&x)[6]) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const bool a = lane & 16, b = lane & 8, c = lane & 4;
+    const T p = add_(a ? x[1] : x[0], __shfl_xor_sync(full, a ? x[0] : x[1], 16));
+    const T q = add_(a ? x[3] : x[2], __shfl_xor_sync(full, a ? x[2] : x[3], 16));
+    const T r = add_(a ? x[5] : x[4], __shfl_xor_sync(full, a ? x[4] : x[5], 16));
+    const T s = add_(b ? q : p, __shfl_xor_sync(full, b ? p : q, 8));
+    const T t = add_(r, __shfl_xor_sync(full, r, 8));
+    T z = add_(c ? t : s, __shfl_xor_sync(full, c ? s : t, 4));
+    z = add_(z, __shfl_xor_sync(full, z, 2));
+    return add_(z, __shfl_xor_sync(full, z, 1));
+}
+
+// Where warp_sum6 leaves its sums: lanes of the form 4 i but 12 and 28 hold one.
+__device__ __forceinline__ bool sum6_lane(int lane) {
+    return (lane & 3) == 0 && lane != 12 && lane != 28;
+}
+__device__ __forceinline__ int sum6_index(int lane) {
+    return ((lane >> 4) & 1) | ((lane >> 2) & 2) | (lane & 4);
+}
+
 // Sum NQ per-thread values over the block (FP32 warp butterfly, then the
 // warps in a fixed order) and add the block total of quantity q0+q to copy
 // `copy` of the fixed-point accumulators.
@@ -308,19 +373,26 @@ __device__ __forceinline__ void block_accumulate(const T (&v)[NQ], unsigned long
                                                  int copy) {
     __shared__ T red[kBlock / 32][NQ];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (NQ == 5) {
+        const T x[6] = {v[0], v[1], v[2], v[3], v[4], T(0)};
+        const T z = warp_sum6(x);
+        if (sum6_lane(lane) && lane != 20) red[warp][sum6_index(lane)] = z;
+    } else {
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        T x = v[q];
+        for (int q = 0; q < NQ; ++q) {
+            T x = v[q];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) x = add_(x, __shfl_xor_sync(0xffffffffu, x, off));
-        if (lane == 0) red[warp][q] = x;
+            for (int off = 16; off > 0; off >>= 1)
+                x = add_(x, __shfl_xor_sync(0xffffffffu, x, off));
+            if (lane == 0) red[warp][q] = x;
+        }
     }
     __syncthreads();
     if (threadIdx.x < NQ) {
         T s = T(0);
 #pragma unroll
         for (int w = 0; w < kBlock / 32; ++w) s = add_(s, red[w][threadIdx.x]);
-        fx_add(acc_slot(acc, copy, q0 + threadIdx.x), acc + kAccFlag, double(s));
+        fx_add(acc_slot(acc, copy, q0 + threadIdx.x), acc + kAccFlag, s);
     }
     __syncthreads();
 }
@@ -764,7 +836,7 @@ __device__ __forceinline__ void stage_issue(const ProbDesc& pd, int base, int ro
 struct FuseCtl {
     bool fin;
     const int* stop;        // shared memory: the decision stops the solve
-    const double* alpha;    // shared memory: the decided step
+    const void* alpha;      // shared memory: the decided step, in the iterate type
 };
 
 // Outcomes of passA_staged.
@@ -787,6 +859,7 @@ __device__ __forceinline__ int passA_staged(const ProbDesc& pd, int r_begin, int
     const T om = om_of<T>(pd);
     T oma = sub_(T(1), alpha);
     const bool greedy = pd.oracle == 0;
+    const T floor_u = greedy ? T(0) : -inf_<T>();   // admissible classes: u > floor_u
     const int stage_elems = 3 * KMAX * kBlock;
     int rc = kPassOk;
     // with fc.fin the caller has issued the first sub-tile's copies and taken
@@ -837,15 +910,17 @@ __device__ __forceinline__ int passA_staged(const ProbDesc& pd, int r_begin, int
                     phases ^= 1u << (buf ^ 1);
                 return kPassStopped;
             }
-            alpha = T(*fc.alpha);
+            alpha = *static_cast<const T*>(fc.alpha);
             oma = sub_(T(1), alpha);
         }
         if (t < rows) {
             const int sp = sv & 0x7f;
             const bool mv = (sv & kActiveBit) != 0;
-            bool binary = true;
+            // rows that stay: u = 1 u + 0; moved rows: fma(oma, u, 0) is oma u
+            const T um = mv ? oma : T(1), ua = mv ? alpha : T(0);
+            bool one = false;
             T best = inf_<T>();
-            int s = -1, first_adm = -1, first_one = -1;
+            int s = -1;
 #pragma unroll
             for (int k = 0; k < KMAX; ++k) {
                 if (k < K) {
@@ -855,36 +930,55 @@ __device__ __forceinline__ int passA_staged(const ProbDesc& pd, int r_begin, int
                         lu = fma_(alpha, sS[k * kBlock + t], mul_(oma, lu));
                         LUb[k * np + r] = lu;
                         sL[k * kBlock + t] = lu;
-                        if (mv) {
-                            u = (k == sp) ? fma_(oma, u, alpha) : mul_(oma, u);
-                            Ub[k * np + r] = u;
-                            sU[k * kBlock + t] = u;
-                        }
+                        u = fma_(um, u, k == sp ? ua : T(0));
+                        if (mv) Ub[k * np + r] = u;
+                        sU[k * kBlock + t] = u;
                     }
-                    binary = binary && (u == T(0) || u == T(1));
-                    if (first_one < 0 && u == T(1)) first_one = k;
-                    T gk = fma_(-c2, u, lu);
-                    if (f >= 0) gk = fma_(om, sub_(u, k == f ? T(1) : T(0)), gk);
-                    const bool adm = !greedy || u > T(0);
-                    if (adm && first_adm < 0) first_adm = k;
-                    if (adm && gk < best) {
+                    one = one || u == T(1);
+                    const T gk = fma_(-c2, u, lu);
+                    if (u > floor_u && gk < best) {
                         best = gk;
                         s = k;
                     }
                 }
             }
-            const bool active = greedy ? !binary : true;
+            // a row is binary only if one of its entries is 1
+            bool binary = false;
+            int at = 0;
+            if (one) {
+                binary = true;
+                for (int k = K - 1; k >= 0; --k) {
+                    const T u = sU[k * kBlock + t];
+                    binary = binary && (u == T(0) || u == T(1));
+                    if (u == T(1)) at = k;
+                }
+            }
+            const bool active = !(greedy && binary);
             T gs = best;
             if (active) {
+                if (f >= 0) {   // labelled rows: the fidelity term of G'
+                    gs = inf_<T>();
+                    s = -1;
+                    for (int k = 0; k < K; ++k) {
+                        const T u = sU[k * kBlock + t];
+                        const T gk = fma_(om, sub_(u, k == f ? T(1) : T(0)),
+                                          fma_(-c2, u, sL[k * kBlock + t]));
+                        if (u > floor_u && gk < gs) {
+                            gs = gk;
+                            s = k;
+                        }
+                    }
+                }
                 if (s < 0) {   // no finite candidate: the gap becomes NaN
-                    s = first_adm < 0 ? 0 : first_adm;
+                    s = 0;
+                    for (int k = K - 1; k >= 0; --k)
+                        if (sU[k * kBlock + t] > floor_u) s = k;
                     gs = CUDART_NAN_F;
                 }
             } else {
-                s = first_one < 0 ? 0 : first_one;
+                s = at;
             }
-            const bool at_vertex = binary && sU[s * kBlock + t] == T(1);
-            const bool moved = active && !at_vertex;
+            const bool moved = active && !(binary && sU[s * kBlock + t] == T(1));
             T gap = T(0), nD = T(0), tLU = T(0);
             if (moved) {
 #pragma unroll

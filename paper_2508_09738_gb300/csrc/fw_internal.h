@@ -53,6 +53,11 @@ public:
     virtual void reinit(const ProbDesc& pd, cudaStream_t s) = 0;
     virtual void labels(const ProbDesc& pd, int32_t* out, cudaStream_t s) = 0;
     virtual void objective(const ProbDesc& pd, const void* LUf, double* part, cudaStream_t s) = 0;
+    // Whether pass B has a form for pattern problems of K classes, and the
+    // search for the patterns of n rows (col: kPatRow 16-bit offsets each).
+    virtual bool pattern_kernels(int K) const = 0;
+    virtual void patterns(int n, const void* col, unsigned long long* keys, int* rep, uint8_t* pat,
+                          int16_t* ptab, int* fail, cudaStream_t s) = 0;
     virtual cudaError_t configure() = 0;   // dynamic shared-memory limits
     // Dynamic shared memory of k_passB_tab for this many lanes per row and
     // rows; 0 when the instantiation has no such form (FP64 iterate, K > 16).
@@ -118,6 +123,7 @@ struct ProbLayout {
     int64_t n = 0, nnz = 0, nnz_pad = 0, npad = 0;
     int32_t K = 0, tile_rows = 0, ntiles = 0, lanes = 1;
     int32_t maxrow = 0;    // entries of the longest row
+    int32_t padw = kPadW;  // rows padded to a multiple of this many entries
     // keep the 4-bit class array (ProbDesc::cls4): set by the two-kernel
     // single-problem path for K <= 16; the persistent kernels do not use it
     bool cls4 = false;

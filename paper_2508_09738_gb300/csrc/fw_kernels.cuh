@@ -1,20 +1,53 @@
 // __global__ kernels of the single-problem path and of graph assembly.
 #pragma once
-#include "fw_device.cuh"
+#include "fw_step.cuh"
 
 namespace fw {
 
 // ---------------------------------------------------------------- hot loop
+// The previous iteration's decision as the blocks of a fused pass A need it
+// (warp 0 of each): the step *alpha, or true when the solve stops.  quick_step
+// where it decides, else the full decision; nothing is committed.
+template <typename T>
+__device__ __forceinline__ bool fused_step(const ProbDesc& pd, ProbState* st, int c, T* alpha) {
+    const unsigned long long* accb = pd.acc + c * kAccBank;
+    if constexpr (sizeof(T) == 4) {
+        const int lane = threadIdx.x & 31;
+        const ulonglong2* S = reinterpret_cast<const ulonglong2*>(accb);
+        ulonglong2 v = __ldcg(S + min(lane, kNumR - 1));
+        const ulonglong2 nW = __ldcg(S + 2), tLU = __ldcg(S + 3);
+        const bool flag = __ldcg(accb + kAccFlag) != 0ull || __ldcg(&st->err) != 0;
+        const double g0 = __ldcg(&st->in[c].g0);
+        const int iter = __ldcg(&st->in[c].iter), g0_set = __ldcg(&st->in[c].g0_set);
+        if (lane == 6) {   // S5 - S3 + S2; v is S5
+            add128(v.x, v.y, ~tLU.x, ~tLU.y);
+            add128(v.x, v.y, 1ull, 0ull);
+            add128(v.x, v.y, nW.x, nW.y);
+        }
+        float af;
+        if (g0_set && quick_step(v.x, v.y, flag, iter, quick_cfg(step_cfg(pd), g0), af)) {
+            *alpha = af;
+            return false;
+        }
+    }
+    double a;
+    const int stop = warp_decide(accb, st, c, step_cfg(pd), false, &a);
+    *alpha = T(a);
+    return stop != 0;
+}
+
 // Step pass A of one tile (k_passA, k_passA_exact).  With `fin` the block first
 // takes the previous iteration's step decision itself (no k_finish between
 // the passes; see ProbState); otherwise it applies the step k_finish stored.
 // `tile`: the problem's row tile this block works on (its block index in the
-// single-problem launch, its work item's tile in a batched item launch).
+// single-problem launch, its work item's tile in a batched item launch).  A
+// fused launch has one block more, with no tile (tile == ntiles): it takes the
+// decision in full and commits it, so that no block with rows waits for FP64.
 template <typename T, int KMAX, bool EXACT>
 __device__ __forceinline__ void passA_step(const ProbDesc& pd, ProbState* st, int fin, T* stage,
                                            int tile) {
     __shared__ __align__(8) uint64_t bars[2];
-    __shared__ double s_alpha;
+    __shared__ T s_alpha;
     __shared__ int s_stop, s_done, s_cur;
     // Block 0 of this launch may commit a stop (done = 1) while other blocks
     // start: one thread reads the flag (and the parity) and the whole block
@@ -28,7 +61,8 @@ __device__ __forceinline__ void passA_step(const ProbDesc& pd, ProbState* st, in
         if (!d) {
             mbar_init(&bars[0], 1);
             mbar_init(&bars[1], 1);
-            if (fin) {   // the first copies go out at once (a step is always pending)
+            if (tile == pd.ntiles) {
+            } else if (fin) {   // the first copies go out at once (a step is always pending)
                 const int r0 = tile * pd.tile_rows;
                 stage_issue<T, KMAX>(pd, r0, min(kBlock, pd.n - r0), true, stage, &bars[0]);
             } else if (tile == 0) {
@@ -39,11 +73,16 @@ __device__ __forceinline__ void passA_step(const ProbDesc& pd, ProbState* st, in
     __syncthreads();
     if (s_done) return;
     const int c = s_cur;
+    if (tile == pd.ntiles) {
+        double a;
+        if (threadIdx.x < 32) warp_decide(pd.acc + c * kAccBank, st, c, step_cfg(pd), true, &a);
+        return;
+    }
     if (fin && threadIdx.x < 32) {
         // warp 0 takes the previous iteration's decision while the copies are
-        // in flight; block 0 commits it
-        double a;
-        const int stop = warp_decide(pd.acc + c * kAccBank, st, c, step_cfg(pd), tile == 0, &a);
+        // in flight
+        T a;
+        const bool stop = fused_step<T>(pd, st, c, &a);
         if (threadIdx.x == 0) {
             s_stop = stop;
             s_alpha = a;
@@ -230,7 +269,142 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_passB_tab(ProbDesc pd, ProbS
 #pragma unroll
         for (int w = 0; w < kBlock / 32; ++w) sum = add_(sum, s_part[threadIdx.x * (kBlock / 32) + w]);
         fx_add(acc_slot(accb, (t0 + int(threadIdx.x)) % kAccCopies, kNumA), accb + kAccFlag,
-               double(sum));
+               sum);
+    }
+}
+
+// Eight weights of a row of a pattern problem: one 256-bit load (FP32; it may
+// leave L2 first, the iterate arrays are read again sooner) or one 128-bit
+// load (BF16).
+__device__ __forceinline__ void ld_w8(const float* p, float (&v)[8]) {
+    asm volatile("ld.global.nc.L1::no_allocate.L2::evict_first.v8.f32 "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]),
+                   "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+}
+__device__ __forceinline__ void ld_w8(const __nv_bfloat16* p, float (&v)[8]) {
+    const int4 t = ld_stream(reinterpret_cast<const int4*>(p));
+    const int w[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        v[2 * i] = __uint_as_float(uint32_t(w[i]) << 16);
+        v[2 * i + 1] = __uint_as_float(uint32_t(w[i]) & 0xffff0000u);
+    }
+}
+
+// a += v where c holds (a predicated add: written with a branch, the compiler
+// turns sums selected by a class into an array indexed by it, in local memory).
+__device__ __forceinline__ void add_if(float& a, bool c, float v) {
+    asm("{\n .reg .pred p;\n setp.ne.s32 p, %1, 0;\n @p add.rn.f32 %0, %0, %2;\n}"
+        : "+f"(a)
+        : "r"(int(c)), "f"(v));
+}
+
+// Pass B of a pattern problem (ProbDesc::pat): one lane per row, exactly K <= 8
+// classes, every row kPatRow slots.  A row's columns follow from its pattern
+// byte, so neither row offsets nor columns are read (images: 21% of pass B's
+// bytes); its weights are one load and its class sums stay in registers (the
+// same sums in the same order as csr_bins).  Each block takes whole row
+// tiles, kPatSubs 256-row sub-tiles side by side; the threads' <D, L S> of up
+// to kPatGroup sub-tiles wait in shared memory and are added in ascending
+// order, as passB_rows adds them, so the sub-tiles themselves run in descending
+// order: pass A has just written the last ones, and the next pass A starts with
+// the first ones, so each finds part of its rows in L2.
+constexpr int kPatThreads = 512;
+constexpr int kPatSubs = kPatThreads / kBlock;
+constexpr int kPatGroup = 16;
+template <typename WT, int K>
+__global__ void __launch_bounds__(kPatThreads, 2) k_passB_pat(ProbDesc pd, ProbState* st) {
+    __shared__ __align__(16) int16_t s_tab[kPatterns][kPatRow];
+    __shared__ float s_q[kPatGroup][kBlock];
+    __shared__ float s_red[kBlock / 32];
+    bool done;
+    unsigned long long* accb = passB_bank(pd, st, done, blockIdx.x);   // block 0 holds tile 0
+    if (done) return;
+    const int tid = threadIdx.x, t = tid & (kBlock - 1), sub = tid / kBlock;
+    if (tid < kPatterns * kPatRow / 8)
+        reinterpret_cast<uint4*>(s_tab)[tid] = __ldg(reinterpret_cast<const uint4*>(pd.ptab) + tid);
+    __syncthreads();
+    const int64_t np = pd.npad;
+    const float* __restrict__ Ub = static_cast<const float*>(pd.U);
+    float* __restrict__ LSb = static_cast<float*>(pd.LS);
+    const float* __restrict__ diag = static_cast<const float*>(pd.diag);
+    const WT* __restrict__ val = static_cast<const WT*>(pd.val);
+    const uint8_t* __restrict__ choice = pd.choice;
+    const int n = pd.n;
+    for (int tile = blockIdx.x; tile < pd.ntiles; tile += gridDim.x) {
+        const int r0 = tile * pd.tile_rows, r1 = min(n, r0 + pd.tile_rows);
+        const int subs = (r1 - r0 + kBlock - 1) / kBlock;
+        float accq = 0.f;   // threads below kBlock: their rows' sum so far
+        for (int g0 = 0; g0 < subs; g0 += kPatGroup) {
+            const int cnt = min(kPatGroup, subs - g0);
+            int j = cnt - 1 - sub;   // this thread's sub-tile of the group
+            int r = r0 + (g0 + j) * kBlock + t;
+            int pid = j >= 0 && r < r1 ? int(__ldg(pd.pat + r)) : 0;
+            for (; j >= 0; j -= kPatSubs) {
+                const bool in = r < r1;
+                const int rn = r - kPatSubs * kBlock;
+                float q = 0.f;
+                int pid_next = 0;
+                if (in) {
+                    float w[kPatRow], u[K];
+                    ld_w8(val + int64_t(r) * kPatRow, w);
+                    const uint8_t sv = __ldg(choice + r);
+#pragma unroll
+                    for (int k = 0; k < K; ++k) u[k] = ld_cg(Ub + k * np + r);
+                    if (j >= kPatSubs) pid_next = __ldg(pd.pat + rn);   // the row below is in range
+                    const uint4 o4 = *reinterpret_cast<const uint4*>(s_tab[pid]);
+                    const uint32_t ow[4] = {o4.x, o4.y, o4.z, o4.w};
+                    int s[kPatRow];
+#pragma unroll
+                    for (int i = 0; i < kPatRow; ++i) {
+                        const int off = i & 1 ? int(ow[i / 2]) >> 16 : int(ow[i / 2] << 16) >> 16;
+                        s[i] = __ldg(choice + uint32_t(r + off)) & 0x7f;
+                    }
+                    float b[K];
+#pragma unroll
+                    for (int k = 0; k < K; ++k) b[k] = 0.f;
+#pragma unroll
+                    for (int i = 0; i < kPatRow; ++i)
+#pragma unroll
+                        for (int k = 0; k < K; ++k)
+                            add_if(b[k], s[i] == k, w[i]);
+                    const int si = sv & 0x7f;
+                    const float dg = pd.comb ? __ldg(diag + r) : 1.f;
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {
+                        const float ls = k == si ? sub_(dg, b[k]) : -b[k];
+                        LSb[k * np + r] = ls;
+                        q = fma_(sub_(k == si ? 1.f : 0.f, u[k]), ls, q);
+                    }
+                    if (!(sv & kActiveBit)) q = 0.f;
+                } else if (j >= kPatSubs) {
+                    pid_next = __ldg(pd.pat + rn);
+                }
+                s_q[j][t] = q;
+                pid = pid_next;
+                r = rn;
+            }
+            __syncthreads();
+            if (sub == 0)
+                for (int i = 0; i < cnt; ++i) accq = add_(accq, s_q[i][t]);
+            __syncthreads();
+        }
+        // the tile's total: butterfly and warp order of block_accumulate
+        if (sub == 0) {
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1)
+                accq = add_(accq, __shfl_xor_sync(0xffffffffu, accq, off));
+            if ((tid & 31) == 0) s_red[tid >> 5] = accq;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            float sum = 0.f;
+#pragma unroll
+            for (int w = 0; w < kBlock / 32; ++w) sum = add_(sum, s_red[w]);
+            fx_add(acc_slot(accb, tile % kAccCopies, kNumA), accb + kAccFlag, sum);
+        }
     }
 }
 
@@ -402,6 +576,59 @@ __global__ void k_build(int64_t n, const int32_t* rp, const int32_t* col, const 
         valp[p] = WT(0.0f);
     }
     if (comb) diag[i] = T(di);
+}
+
+// ------------------------------------------------------- offset patterns
+// Key of a row's offset list (an FNV-style hash of its kPatRow offsets; equal
+// keys are compared offset by offset before they count as equal).  0 marks an
+// empty table entry.
+__device__ __forceinline__ unsigned long long pat_key(const uint4& o) {
+    unsigned long long h = 1469598103934665603ull;
+    const uint32_t w[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) h = (h ^ w[i]) * 1099511628211ull;
+    h ^= h >> 29;
+    return h ? h : 1ull;
+}
+// Collect the distinct offset lists (col: int16 offsets, kPatRow per row) in an
+// open-addressing table; *fail when there are more than the table holds.
+static __global__ void k_pat_find(int n, const int16_t* col, unsigned long long* keys, int* rep,
+                                  int* fail) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= n || *reinterpret_cast<volatile int*>(fail)) return;
+    const unsigned long long key = pat_key(reinterpret_cast<const uint4*>(col)[r]);
+    for (int i = 0, h = int(key % kPatterns); i < kPatterns; ++i, h = (h + 1) % kPatterns) {
+        unsigned long long have = *reinterpret_cast<volatile unsigned long long*>(keys + h);
+        if (have == 0ull) {
+            have = atomicCAS(keys + h, 0ull, key);
+            if (have == 0ull) {
+                rep[h] = r;
+                return;
+            }
+        }
+        if (have == key) return;
+    }
+    *fail = 1;
+}
+// Every row's pattern; *fail when two lists share a key.
+static __global__ void k_pat_assign(int n, const int16_t* col, const unsigned long long* keys,
+                                    const int* rep, uint8_t* pat, int16_t* ptab, int* fail) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint4* rows = reinterpret_cast<const uint4*>(col);
+    if (blockIdx.x == 0 && threadIdx.x < kPatterns)
+        reinterpret_cast<uint4*>(ptab)[threadIdx.x] =
+            keys[threadIdx.x] ? rows[rep[threadIdx.x]] : make_uint4(0, 0, 0, 0);
+    if (r >= n || *fail) return;
+    const uint4 o = rows[r];
+    const unsigned long long key = pat_key(o);
+    for (int i = 0, h = int(key % kPatterns); i < kPatterns; ++i, h = (h + 1) % kPatterns) {
+        if (keys[h] != key) continue;
+        const uint4 p = rows[rep[h]];
+        if (p.x != o.x || p.y != o.y || p.z != o.z || p.w != o.w) *fail = 1;
+        pat[r] = uint8_t(h);
+        return;
+    }
+    *fail = 1;
 }
 
 // U_0 = U_hat (Sec. 5.1): e_c on fidelity rows, 1/K elsewhere; choice reset.

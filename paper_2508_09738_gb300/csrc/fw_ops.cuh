@@ -15,6 +15,8 @@ public:
     static constexpr bool kExactB = sizeof(T) == 4 && KMAX <= 12;
     // 2 / 4 lanes per row, 5..12 classes, FP32 iterate: the 40-register pass B
     static constexpr bool kBound6 = sizeof(T) == 4 && KMAX >= 8 && KMAX <= 12;
+    // pass B of pattern problems: FP32 iterate, class sums in registers
+    static constexpr bool kPat = sizeof(T) == 4 && KMAX <= 8;
     // pass B with the class table in shared memory: FP32 iterate, 4-bit classes
     static constexpr bool kTab = sizeof(T) == 4 && KMAX <= 16;
     size_t elem() const override { return sizeof(T); }
@@ -83,14 +85,14 @@ public:
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem()));
     }
     void passA(const ProbDesc& pd, ProbState* st, cudaStream_t s, int fin) override {
+        const unsigned grid = unsigned(pd.ntiles) + (fin ? 1u : 0u);   // see passA_step
         if constexpr (kExactA) {
             if (pd.K == KMAX) {
-                k_passA_exact<T, KMAX><<<pd.ntiles, kBlock, smemA(pd), s>>>(pd, st, fin);
+                k_passA_exact<T, KMAX><<<grid, kBlock, smemA(pd), s>>>(pd, st, fin);
                 return;
             }
         }
-        k_passA<T, KMAX, MODE_STEP><<<pd.ntiles, kBlock, smemA(pd), s>>>(pd, st, nullptr, nullptr,
-                                                                         fin);
+        k_passA<T, KMAX, MODE_STEP><<<grid, kBlock, smemA(pd), s>>>(pd, st, nullptr, nullptr, fin);
     }
     void flush(const ProbDesc& pd, ProbState* st, cudaStream_t s) override {
         k_passA<T, KMAX, MODE_FLUSH><<<pd.ntiles, kBlock, 0, s>>>(pd, st, nullptr, nullptr, 0);
@@ -128,7 +130,25 @@ public:
         else
             k_passB_tab<T, WT, KMAX, 4, EXACT><<<g, kTabThreads, sm, s>>>(pd, st);
     }
+    template <int K>
+    void passB_pat(const ProbDesc& pd, ProbState* st, cudaStream_t s) {
+        k_passB_pat<WT, K><<<unsigned(pd.pat_grid), kPatThreads, 0, s>>>(pd, st);
+    }
+    bool pattern_kernels(int K) const override { return kPat && K <= KMAX; }
     void passB(const ProbDesc& pd, ProbState* st, cudaStream_t s) override {
+        if constexpr (kPat) {
+            if (pd.pat) {
+                switch (pd.K) {
+                    case 2: if constexpr (KMAX == 4) passB_pat<2>(pd, st, s); return;
+                    case 3: if constexpr (KMAX == 4) passB_pat<3>(pd, st, s); return;
+                    case 4: if constexpr (KMAX == 4) passB_pat<4>(pd, st, s); return;
+                    case 5: if constexpr (KMAX == 8) passB_pat<5>(pd, st, s); return;
+                    case 6: if constexpr (KMAX == 8) passB_pat<6>(pd, st, s); return;
+                    case 7: if constexpr (KMAX == 8) passB_pat<7>(pd, st, s); return;
+                    default: if constexpr (KMAX == 8) passB_pat<8>(pd, st, s); return;
+                }
+            }
+        }
         if constexpr (kTab) {
             if (pd.tab_grid > 0) {   // choose_tab checked lanes, tiles and the fit
                 if (pd.K == KMAX) passB_tab<true>(pd, st, s);
@@ -159,6 +179,13 @@ public:
     }
     void spmm(const ProbDesc& pd, const void* X, void* out, cudaStream_t s) override {
         k_spmm<T, WT, KMAX><<<pd.ntiles, kBlock, smem(), s>>>(pd, (const T*)X, (T*)out);
+    }
+    void patterns(int n, const void* col, unsigned long long* keys, int* rep, uint8_t* pat,
+                  int16_t* ptab, int* fail, cudaStream_t s) override {
+        const unsigned g = unsigned((n + kBlock - 1) / kBlock);
+        k_pat_find<<<g, kBlock, 0, s>>>(n, static_cast<const int16_t*>(col), keys, rep, fail);
+        k_pat_assign<<<g, kBlock, 0, s>>>(n, static_cast<const int16_t*>(col), keys, rep, pat, ptab,
+                                          fail);
     }
     void build(int64_t n, const int32_t* rp, const int32_t* col, const double* w,
                const double* deg, const int32_t* rpp, int32_t* colp, void* valp, void* diag,

@@ -278,31 +278,6 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target) {
 }
 
 // ------------------------------------------------------------------ warps
-// Butterfly sums of six values over a warp with the pairing of
-// block_accumulate (16, 8, 4, 2, 1): at each of the first three steps half of
-// the lanes go on with one value and half with another, so 8 shuffles do the
-// work of 30 and every sum has the same bits.  Lane 0 returns x[0], 16 x[1],
-// 8 x[2], 24 x[3], 4 x[4], 20 x[5].
-template <typename T>
-__device__ __forceinline__ T warp_sum6(const T (&x)[6]) {
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const bool a = lane & 16, b = lane & 8, c = lane & 4;
-    const T p = add_(a ? x[1] : x[0], __shfl_xor_sync(full, a ? x[0] : x[1], 16));
-    const T q = add_(a ? x[3] : x[2], __shfl_xor_sync(full, a ? x[2] : x[3], 16));
-    const T r = add_(a ? x[5] : x[4], __shfl_xor_sync(full, a ? x[4] : x[5], 16));
-    const T s = add_(b ? q : p, __shfl_xor_sync(full, b ? p : q, 8));
-    const T t = add_(r, __shfl_xor_sync(full, r, 8));
-    T z = add_(c ? t : s, __shfl_xor_sync(full, c ? s : t, 4));
-    z = add_(z, __shfl_xor_sync(full, z, 2));
-    return add_(z, __shfl_xor_sync(full, z, 1));
-}
-
-__device__ __forceinline__ void add128(unsigned long long& lo, unsigned long long& hi,
-                                       unsigned long long l2, unsigned long long h2) {
-    lo += l2;
-    hi += h2 + (lo < l2 ? 1ull : 0ull);
-}
 // 128-bit sums over the lanes l, l ^ off, l ^ off/2, ... down to l ^ last
 template <int OFF, int LAST>
 __device__ __forceinline__ void warp_sum128(unsigned long long& lo, unsigned long long& hi) {
@@ -890,10 +865,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
                 if (f >= 0) x[2] = fma_(om, x[1], T(0));
             }
             const T z = warp_sum6(x);
-            if ((lane & 3) == 0 && lane != 12 && lane != 28) {
-                const int q = ((lane >> 4) & 1) | ((lane >> 2) & 2) | (lane & 4);
-                s_part[q][u0] = z;
-            }
+            if (sum6_lane(lane)) s_part[sum6_index(lane)][u0] = z;
         }
         __syncthreads();
         ResSlot* const tot = s_ring[it % kResRing];

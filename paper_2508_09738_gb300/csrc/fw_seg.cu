@@ -199,6 +199,37 @@ static fw_status plan_resident(fw_seg* h) {
     return FW_OK;
 }
 
+// Find the offset patterns of a regular grid, for the pass B that reads no
+// columns.  Not for problems the resident kernel takes, nor when the caller
+// asks for a pass B form.
+static fw_status plan_patterns(fw_seg* h) {
+    const ProbLayout& lay = h->lay;
+    if (h->res_plan.group > 0 || h->opts.class_table != FW_TABLE_AUTO || h->pd.tab_grid > 0 ||
+        lay.padw != kPatRow || !h->pd.col16 || h->pd.lanes != 1 ||
+        !h->ops->pattern_kernels(lay.K))
+        return FW_OK;
+    uint8_t* pat = nullptr;
+    if (h->alloc(&pat, (size_t(lay.n) + 255) / 256 * 256 + kPatterns * kPatRow * 2) != FW_OK)
+        return FW_OK;
+    int16_t* ptab = reinterpret_cast<int16_t*>(pat + (size_t(lay.n) + 255) / 256 * 256);
+    Temps t(h->stream);
+    unsigned long long* keys = nullptr;
+    FW_TRY(t.get(&keys, 12 * kPatterns + 16));
+    int* rep = reinterpret_cast<int*>(keys + kPatterns);
+    FW_CUDA(cudaMemsetAsync(keys, 0, 12 * kPatterns + 16, h->stream));
+    h->ops->patterns(h->pd.n, h->pd.col, keys, rep, pat, ptab, rep + kPatterns, h->stream);
+    FW_TRY(launch_check("pattern kernels"));
+    int fail = 0, sms = 0;
+    FW_CUDA(cudaMemcpyAsync(&fail, rep + kPatterns, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    FW_CUDA(cudaStreamSynchronize(h->stream));
+    if (fail) return FW_OK;
+    FW_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    h->pd.pat = pat;
+    h->pd.ptab = ptab;
+    h->pd.pat_grid = std::min(h->pd.ntiles, 2 * sms);   // two 512-thread blocks per SM
+    return FW_OK;
+}
+
 // Up to `iters` iterations in one resident launch (it ends at the stop rule).
 static fw_status launch_resident(fw_seg* h, int iters) {
     FW_CUDA(res_launch(h->res.get(), h->res_args, h->res_plan, iters, h->stream));
@@ -439,6 +470,7 @@ fw_status fw_seg_create(fw_seg** out, int64_t n, const int32_t* row_ptr, const i
         FW_TRY(assemble_uploaded(h->ops.get(), *up, lay, h->pd, h->st, h->stream));
         up.reset();   // its device copies go back to the pool
         FW_TRY(plan_resident(h.get()));
+        FW_TRY(plan_patterns(h.get()));
         FW_TRY(read_state(h.get()));
         if (h->res_plan.group == 0 && build_graph(h.get()) != FW_OK) {
             // streams that cannot be captured (the legacy default stream) run

@@ -76,13 +76,13 @@ __global__ void __launch_bounds__(kBlock) k_state_init(ProbState* st, const doub
     }
 }
 
-// Padded row offsets (every row rounded up to kPadW entries), an exclusive
+// Padded row offsets (every row rounded up to padw entries), an exclusive
 // scan over the rows in three steps: per 1024-row block, over the block
 // totals (one block), then the block offsets added back.  Integer, so exact.
 constexpr int kScanRows = 4 * kBlock;
 
 __global__ void __launch_bounds__(kBlock)
-k_pad_scan_local(int64_t n, const int32_t* __restrict__ rp, int32_t* __restrict__ out,
+k_pad_scan_local(int64_t n, int padw, const int32_t* __restrict__ rp, int32_t* __restrict__ out,
                  int32_t* __restrict__ bsum) {
     __shared__ int32_t wsum[kBlock / 32];
     const int64_t base = blockIdx.x * int64_t(kScanRows) + threadIdx.x * 4;
@@ -93,7 +93,7 @@ k_pad_scan_local(int64_t n, const int32_t* __restrict__ rp, int32_t* __restrict_
     for (int q = 0; q < 4; ++q) {
         const int64_t i = base + q;
         const int32_t d = i < n ? rp[i + 1] - rp[i] : 0;
-        v[q] = (d + (kPadW - 1)) & ~(kPadW - 1);
+        v[q] = (d + (padw - 1)) & ~(padw - 1);
         s += v[q];
     }
     int32_t x = s;
@@ -348,6 +348,14 @@ fw_status plan_problem(const HostGraph& g, const fw_seg_opts& o, ProbLayout& lay
     if (bad) return invalid("labels must be -1 or in [0, K)");
     lay.n = n;
     lay.nnz = g.rp[n];
+    // Rows of 5 to 8 entries nearly everywhere (pixel grids): eight slots for
+    // each, so that row r's entries start at 8 r (see k_passB_pat)
+    lay.padw = kPadW;
+    if (longest > 4 && longest <= kPatRow && o.index_width != 32 && lay.nnz >= 5 * n &&
+        double(kPatRow) * double(n) <= 1.02 * double(acc) && kPatRow * n < int64_t(1) << 31) {
+        lay.padw = kPatRow;
+        acc = kPatRow * n;
+    }
     lay.nnz_pad = acc;
     lay.maxrow = int32_t(longest);
     if (lay.nnz > 0 && (!g.col || !g.w)) return invalid("col and w must not be NULL");
@@ -584,7 +592,7 @@ fw_status assemble_uploaded(Ops* ops, Upload& up, const ProbLayout& lay, ProbDes
         int32_t* d_bsum = nullptr;
         FW_TRYS(t.get(&d_bsum, 4 * size_t(nb)));
         int32_t* prp = const_cast<int32_t*>(pd.rp);
-        k_pad_scan_local<<<nb, kBlock, 0, s>>>(n, d_rp, prp, d_bsum);
+        k_pad_scan_local<<<nb, kBlock, 0, s>>>(n, lay.padw, d_rp, prp, d_bsum);
         k_pad_scan_blocks<<<1, kBlock, 0, s>>>(n, nb, d_bsum, prp);
         k_pad_scan_add<<<unsigned((n + kBlock - 1) / kBlock), kBlock, 0, s>>>(n, d_bsum, prp);
         FW_TRYS(launched("row offset scan"));

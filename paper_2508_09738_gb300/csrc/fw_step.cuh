@@ -7,37 +7,6 @@
 
 namespace fw {
 
-// Q64.64 of a tile total in the iterate type, the value fx_split gives for
-// double(v).  An FP32 total is shifted into place with integer instructions;
-// small negative ones (whose 1 - frac rounds in FP64) and large ones take
-// fx_split itself.
-__device__ __forceinline__ bool fx_total_split(double v, unsigned long long& lo,
-                                               unsigned long long& hi) {
-    return fx_split(v, lo, hi);
-}
-__device__ __forceinline__ bool fx_total_split(float v, unsigned long long& lo,
-                                               unsigned long long& hi) {
-    const uint32_t b = __float_as_uint(v);
-    const int ex = int((b >> 23) & 0xff);
-    const bool neg = (b >> 31) != 0;
-    // |v| < 2^40, and |v| >= 2^-29 when negative (then 1 - frac is exact)
-    if (ex >= 127 + 40 || (neg && ex < 127 - 29 && (b << 1) != 0u)) return fx_split(double(v), lo, hi);
-    const unsigned long long m = ex ? ((b & 0x7fffffu) | 0x800000u) : (b & 0x7fffffu);
-    const int sh = (ex ? ex : 1) - 150 + 64;   // v = m 2^(sh - 64)
-    if (sh >= 0) {
-        lo = sh < 64 ? m << sh : 0ull;
-        hi = sh >= 64 ? m << (sh - 64) : (sh > 40 ? m >> (64 - sh) : 0ull);
-    } else {
-        lo = sh > -64 ? m >> -sh : 0ull;
-        hi = 0ull;
-    }
-    if (neg) {
-        lo = ~lo + 1ull;
-        hi = ~hi + (lo == 0ull ? 1ull : 0ull);
-    }
-    return true;
-}
-
 // A positive value as (h + l) 2^e with h in [1, 2) and l in [0, 2^-23): 46
 // bits, cut off below.
 struct Pair {
@@ -80,18 +49,22 @@ struct QuickCfg {
     int tol_mode;     // 0: no threshold (gap_tol = 0), 1: tol holds it, 2: not representable here
     int armijo, max_iters;
 };
-__device__ __forceinline__ bool pair_range(double v) {   // normal, well inside the float exponents
-    const int ex = int((static_cast<unsigned long long>(__double_as_longlong(v)) >> 52) & 0x7ff);
-    return v > 0.0 && ex > 1023 - 100 && ex < 1023 + 100;
+__device__ __forceinline__ bool pair_range(double v) {   // positive, well inside the float exponents
+    const int ex = int(static_cast<unsigned long long>(__double_as_longlong(v)) >> 52);   // sign included
+    return ex > 1023 - 100 && ex < 1023 + 100;
 }
 __device__ __forceinline__ QuickCfg quick_cfg(const StepCfg& cfg, double g0) {
     QuickCfg q;
-    const double c2 = 2.0 * cfg.inv_eps;
-    q.has_c2 = c2 == 0.0 ? 0 : pair_range(c2) ? 1 : 2;
-    q.c2 = pair_of_double(c2);
-    const double tol = cfg.tol_mode ? cfg.gap_tol * g0 : cfg.gap_tol;
-    q.tol_mode = cfg.gap_tol == 0.0 ? 0 : pair_range(tol) ? 1 : 2;
-    q.tol = pair_of_double(tol);
+    q.has_c2 = !positive_bits(cfg.inv_eps) ? 0 : pair_range(cfg.inv_eps) ? 1 : 2;
+    q.c2 = pair_of_double(cfg.inv_eps);
+    ++q.c2.e;
+    q.tol_mode = 0;
+    q.tol = q.c2;
+    if (positive_bits(cfg.gap_tol)) {
+        const double tol = cfg.tol_mode ? cfg.gap_tol * g0 : cfg.gap_tol;
+        q.tol_mode = pair_range(tol) ? 1 : 2;
+        q.tol = pair_of_double(tol);
+    }
     q.armijo = cfg.step_rule;
     q.max_iters = cfg.max_iters;
     return q;

@@ -10,6 +10,11 @@ constexpr int kTilesTarget = 1216;  // a problem has at most this many row tiles
 constexpr int kNumA = 5;            // row-pass partials: g, ||D||^2, sum w||D||^2, <D,LU>, |I|
 constexpr int kNumB = 1;            // CSR-pass partial: <D, L S>
 constexpr int kNumR = kNumA + kNumB;  // accumulated quantities (pass A 0..4, pass B 5)
+// Offset patterns of regular grids: a row is one of at most kPatterns lists of
+// column offsets (pixel grids have one for interior rows and one for each edge
+// and corner), with exactly kPatRow entry slots per row.
+constexpr int kPatterns = 64;
+constexpr int kPatRow = 8;
 constexpr uint8_t kActiveBit = 0x80;  // bit 7 of the choice byte: row moved by the oracle
 // Exact tile-total accumulators: kAccCopies copies of the kNumR Q64.64
 // quantities (lo, hi words, kAccLine words apart), then a non-finite flag.
@@ -44,6 +49,8 @@ struct ProbDesc {
     uint8_t* cls4;       // [(n+1)/2] the same classes as 4-bit pairs (row 2m low nibble,
                          // 2m+1 high) for K <= 16, gathered by pass B; NULL for K > 16
     const int8_t* fid;   // [n] fidelity class or -1
+    const uint8_t* pat;  // [n] row's offset pattern, or NULL (pass B reads col)
+    const int16_t* ptab; // [kPatterns][8] the patterns' column offsets j - i (padding: 0)
     unsigned long long* acc;  // [kAccTotal]: two banks of kAccWords Q64.64 totals (see
                               // kAccCopies) and a non-finite flag; exact and order-free
     int32_t n;           // rows
@@ -60,6 +67,8 @@ struct ProbDesc {
     int32_t col16;       // 1: col holds 16-bit offsets (every |j - i| < 2^15)
     int32_t tab_grid;    // > 0: pass B runs k_passB_tab on this many blocks (class table
                          // in shared memory); 0: the direct pass-B kernels
+    int32_t pat_grid;    // blocks of k_passB_pat
+    int32_t pad_;
     int32_t band;        // largest |j - i| of the stored entries
     double inv_eps;      // 1/eps (0 when eps = +inf)
     double omega0;       // fidelity weight
