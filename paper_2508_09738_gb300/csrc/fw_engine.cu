@@ -834,16 +834,14 @@ public:
     }
 
     fw_status get_U(int s, double* out) {
-        const Slot& sl = slots[size_t(s)];
-        const size_t np = size_t(sl.lay.npad), K = size_t(sl.lay.K), n = size_t(sl.lay.n);
-        std::vector<unsigned char> tmp(te * np * K);
-        FW_CUDA(cudaMemcpyAsync(tmp.data(), sl.pd.U, tmp.size(), cudaMemcpyDeviceToHost, stream));
-        FW_CUDA(cudaStreamSynchronize(stream));
-        for (size_t i = 0; i < n; ++i)
-            for (size_t k = 0; k < K; ++k)
-                out[i * K + k] = te == 4 ? double(reinterpret_cast<float*>(tmp.data())[k * np + i])
-                                         : reinterpret_cast<double*>(tmp.data())[k * np + i];
-        return FW_OK;
+        const ProbLayout& lay = slots[size_t(s)].lay;
+        Temps t(stream);
+        void* scratch = nullptr;
+        const size_t row = sizeof(double) * size_t(lay.K);
+        const size_t bytes = std::max(row * kRmRows, std::min(row * size_t(lay.n), size_t(8) << 20));
+        FW_TRY(t.get(&scratch, bytes));
+        return rowmajor_to_host(ops.get(), slots[size_t(s)].pd.U, lay.n, lay.npad, lay.K, out,
+                                scratch, bytes, stream);
     }
 };
 

@@ -51,6 +51,9 @@ public:
                        const double* deg, const int32_t* rpp, int32_t* colp, void* valp,
                        void* diag, int comb, int col16, cudaStream_t s) = 0;
     virtual void reinit(const ProbDesc& pd, cudaStream_t s) = 0;
+    // out[(i - r0) K + k] = X[k npad + i] for rows i of [r0, r0 + rows)
+    virtual void rowmajor(const void* X, int64_t npad, int K, int64_t r0, int64_t rows, double* out,
+                          cudaStream_t s) = 0;
     virtual void labels(const ProbDesc& pd, int32_t* out, cudaStream_t s) = 0;
     virtual void objective(const ProbDesc& pd, const void* LUf, double* part, cudaStream_t s) = 0;
     // Whether pass B has a form for pattern problems of K classes, and the
@@ -164,6 +167,12 @@ struct Temps {
         return FW_OK;
     }
 };
+
+// Copy a class-major array X[K][npad] (n rows) to the host as row-major doubles;
+// `scratch` (device, `bytes` long) holds as many rows at a time as it can.
+// Waits for the stream.
+fw_status rowmajor_to_host(Ops* ops, const void* X, int64_t n, int64_t npad, int K, double* out,
+                           void* scratch, size_t bytes, cudaStream_t s);
 
 // Device copies of a caller's input arrays (row_ptr, col, w, labels).
 struct Upload {

@@ -476,6 +476,26 @@ __global__ void k_labels(ProbDesc pd, int32_t* out) {
     out[r] = b;
 }
 
+// Rows [r0, r0 + rows) of a class-major array as row-major doubles, 64 rows a
+// block: read a class at a time, written as one contiguous run.
+constexpr int kRmRows = 64;
+template <typename T>
+__global__ void __launch_bounds__(kBlock) k_rowmajor(const T* X, int64_t npad, int K, int64_t r0,
+                                                     int64_t rows, double* out) {
+    __shared__ T s[32 * (kRmRows + 1)];
+    const int64_t b = blockIdx.x * int64_t(kRmRows);
+    const int cnt = rows - b < kRmRows ? int(rows - b) : kRmRows;
+    for (int e = threadIdx.x; e < K * kRmRows; e += kBlock) {
+        const int k = e / kRmRows, i = e % kRmRows;
+        if (i < cnt) s[k * (kRmRows + 1) + i] = X[k * npad + r0 + b + i];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < cnt * K; e += kBlock) {
+        const int i = e / K, k = e - i * K;
+        out[b * K + e] = double(s[k * (kRmRows + 1) + i]);
+    }
+}
+
 // Per-block FP64 partials of E(U) with a freshly computed LUf = L U
 // (eq. gradgl_vv2): 1/2 <U, L U> + 1/eps sum u(1-u) + 1/2 sum w_i ||u_hat_i - u_i||^2.
 template <typename T>

@@ -197,6 +197,11 @@ public:
     void reinit(const ProbDesc& pd, cudaStream_t s) override {
         k_reinit<T><<<rows_grid(pd), kBlock, 0, s>>>(pd);
     }
+    void rowmajor(const void* X, int64_t npad, int K, int64_t r0, int64_t rows, double* out,
+                  cudaStream_t s) override {
+        k_rowmajor<T><<<unsigned((rows + kRmRows - 1) / kRmRows), kBlock, 0, s>>>(
+            static_cast<const T*>(X), npad, K, r0, rows, out);
+    }
     void labels(const ProbDesc& pd, int32_t* out, cudaStream_t s) override {
         k_labels<T><<<rows_grid(pd), kBlock, 0, s>>>(pd, out);
     }

@@ -289,6 +289,41 @@ __device__ __forceinline__ void warp_sum128(unsigned long long& lo, unsigned lon
     }
 }
 
+// Tests of the row evaluation.  For FP64 they work on the bits: an FP64
+// compare holds the scheduler for 64 cycles, as any other FP64 instruction.
+__device__ __forceinline__ bool is_one(float u) { return u == 1.0f; }
+__device__ __forceinline__ bool is_one(double u) {
+    return __double_as_longlong(u) == 0x3ff0000000000000ll;
+}
+__device__ __forceinline__ bool is_binary(float u) { return u == 0.0f || u == 1.0f; }
+__device__ __forceinline__ bool is_binary(double u) {
+    return is_one(u) || (__double_as_longlong(u) << 1) == 0ll;
+}
+__device__ __forceinline__ bool is_pos(float u) { return u > 0.0f; }
+__device__ __forceinline__ bool is_pos(double u) {
+    return __double_as_longlong(u) > 0ll && __double_as_longlong(u) <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool less(float a, float b) { return a < b; }
+__device__ __forceinline__ bool less(double a, double b) {   // b is not NaN
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    const long long inf = 0x7ff0000000000000ll, mag = 0x7fffffffffffffffll;
+    // order of the bits with negative values mirrored; -0 counts as +0
+    const long long kx = x < 0 ? -(x & mag) : x, ky = y < 0 ? -(y & mag) : y;
+    return (x & mag) <= inf && kx < ky;
+}
+// L S and D at class k of a row: only the entry of class s takes arithmetic,
+// done once by the caller (ss = diag - b_s, ds = 1 - u_s) where FP64 is slow.
+template <typename T>
+__device__ __forceinline__ T ls_of(bool at, T diag, T bk, T ss) {
+    if constexpr (sizeof(T) == 8) return at ? ss : -bk;
+    else return at ? sub_(diag, bk) : -bk;
+}
+template <typename T>
+__device__ __forceinline__ T d_of(bool at, T u, T ds) {
+    if constexpr (sizeof(T) == 8) return at ? ds : -u;
+    else return sub_(at ? T(1) : T(0), u);
+}
+
 // Four weights as loaded, widened when they are used.
 template <typename WT> struct Weights4;
 template <> struct Weights4<float> {
@@ -492,8 +527,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
     const bool multi = a.cluster && a.group > 1;
     const T* __restrict__ diag = static_cast<const T*>(pd.diag);
     const T c2 = c2_of<T>(pd), om = om_of<T>(pd);
-    const bool greedy = pd.oracle == 0;
-    const T floor_u = greedy ? T(0) : -inf_<T>();           // admissible classes: u > floor_u
+    const bool greedy = pd.oracle == 0;   // admissible classes: u > 0 (greedy), or all
 
     // ------------------------------------------------------- shared memory
     T* const slab = reinterpret_cast<T*>(smraw);            // [layers][K][512]: row sums
@@ -604,14 +638,15 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
                     const bool mv = (meta[r] & kActiveBit) != 0;
                     // rows that stay: u = 1 u + 0; moved rows: fma(oma, u, 0) is oma u
                     const T um = mv ? oma : T(1), ua = mv ? alpha : T(0);
+                    T ss = T(0);
+                    if constexpr (sizeof(T) == 8) ss = sub_(dg, b[sv * kResThreads]);
 #pragma unroll
                     for (int k = 0; k < KMAX; ++k)
                         if (k < K) {
-                            const T bk = b[k * kResThreads];
-                            const T ls = (k == sv) ? sub_(dg, bk) : -bk;
+                            const T ls = ls_of(k == sv, dg, b[k * kResThreads], ss);
                             LU[r][k] = fma_(alpha, ls, mul_(oma, LU[r][k]));
                             U[r][k] = fma_(um, U[r][k], k == sv ? ua : T(0));
-                            one = one || U[r][k] == T(1);
+                            one = one || is_one(U[r][k]);
                         }
                 }
                 // a row is binary only if one of its entries is 1
@@ -624,8 +659,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
                     for (int k = 0; k < KMAX; ++k)
                         if (k < K) {
                             const T u = U[r][k];
-                            binary = binary && (u == T(0) || u == T(1));
-                            if (f1 < 0 && u == T(1)) f1 = k;
+                            binary = binary && is_binary(u);
+                            if (f1 < 0 && is_one(u)) f1 = k;
                         }
                     at = f1 < 0 ? 0 : f1;
                 }
@@ -641,7 +676,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
                             if (k < K) {
                                 const T u = U[r][k];
                                 const T gk = fma_(-c2, u, LU[r][k]);
-                                if (u > floor_u && gk < gs) {
+                                if ((!greedy || is_pos(u)) && less(gk, gs)) {
                                     gs = gk;
                                     s = k;
                                 }
@@ -653,7 +688,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
                                 const T u = U[r][k];
                                 const T gk = fma_(om, sub_(u, k == f ? T(1) : T(0)),
                                                   fma_(-c2, u, LU[r][k]));
-                                if (u > floor_u && gk < gs) {
+                                if ((!greedy || is_pos(u)) && less(gk, gs)) {
                                     gs = gk;
                                     s = k;
                                 }
@@ -662,7 +697,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
                     if (s < 0) {   // no finite candidate: the gap becomes NaN
 #pragma unroll
                         for (int k = KMAX - 1; k >= 0; --k)
-                            if (k < K && U[r][k] > floor_u) s = k;
+                            if (k < K && (!greedy || is_pos(U[r][k]))) s = k;
                         if (s < 0) s = 0;
                         gs = CUDART_NAN_F;
                     }
@@ -671,7 +706,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
                     if (binary) {
 #pragma unroll
                         for (int k = 0; k < KMAX; ++k)
-                            if (k < K && k == s) at_vertex = U[r][k] == T(1);
+                            if (k < K && k == s) at_vertex = is_one(U[r][k]);
                     }
                     meta[r] = (meta[r] & ~0xff) | s | (at_vertex ? 0 : int(kActiveBit));
                 }
@@ -847,15 +882,22 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
                 const int s = meta[r] & 0x7f, f = (meta[r] >> 8) - 1;
                 const T* b = slab + size_t(r) * K * kResThreads + tid;
                 const T dg = pd.comb ? __ldg(diag + row) : T(1);
+                T ss = T(0), ds = T(0);
+                if constexpr (sizeof(T) == 8) {
+                    ss = sub_(dg, b[s * kResThreads]);
+#pragma unroll
+                    for (int k = 0; k < KMAX; ++k)
+                        if (k < K) ds = k == s ? U[r][k] : ds;
+                    ds = sub_(T(1), ds);
+                }
 #pragma unroll
                 for (int k = 0; k < KMAX; ++k)
                     if (k < K) {
                         const T u = U[r][k], lu = LU[r][k];
-                        const T bk = b[k * kResThreads];
                         T gk = fma_(-c2, u, lu);
                         if (f >= 0) gk = fma_(om, sub_(u, k == f ? T(1) : T(0)), gk);
-                        const T d = sub_(k == s ? T(1) : T(0), u);
-                        const T ls = (k == s) ? sub_(dg, bk) : -bk;
+                        const T d = d_of(k == s, u, ds);
+                        const T ls = ls_of(k == s, dg, b[k * kResThreads], ss);
                         x[0] = fma_(u, sub_(gk, best[r]), x[0]);
                         x[1] = fma_(d, d, x[1]);
                         x[3] = fma_(d, lu, x[3]);
@@ -1120,6 +1162,11 @@ public:
             const int c = cluster_of(blocks);
             if (c <= kResMaxCluster && attempt(pd, nt, c, 1, p, maxlen, nnz_pad)) return true;
             if (blocks <= sms && attempt(pd, nt, blocks, 0, p, maxlen, nnz_pad)) return true;
+        }
+        if (sizeof(T) == 8) {   // FP64 issue bounds it: one tile a block, as many SMs as that takes
+            const int ct = cluster_of(nt);
+            if (ct <= kResMaxCluster && attempt(pd, nt, ct, 1, p, maxlen, nnz_pad)) return true;
+            if (nt <= sms && attempt(pd, nt, nt, 0, p, maxlen, nnz_pad)) return true;
         }
         const int c = std::min(kResMaxCluster, cluster_of(pairs)), g = std::min(sms, pairs);
         // A cluster exchanges in 400 cycles what the grid barrier takes 2,300

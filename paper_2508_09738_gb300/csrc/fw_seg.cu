@@ -266,22 +266,20 @@ static fw_status status_of(const ProbState& st) {
     return fw_status(st.status);
 }
 
+// A class-major array of the handle to the host as row-major doubles, through
+// d_tmp, or a few MB of the pool when the array is d_tmp itself.
 static fw_status copy_soa_to_host(fw_seg* h, const void* dev, double* out) {
-    const size_t te = h->ops->elem();
-    const size_t npad = size_t(h->lay.npad), K = size_t(h->lay.K), n = size_t(h->lay.n);
-    std::vector<unsigned char> tmp(te * npad * K);
-    FW_CUDA(cudaMemcpyAsync(tmp.data(), dev, tmp.size(), cudaMemcpyDeviceToHost, h->stream));
-    FW_CUDA(cudaStreamSynchronize(h->stream));
-    if (te == 4) {
-        const float* t = reinterpret_cast<const float*>(tmp.data());
-        for (size_t i = 0; i < n; ++i)
-            for (size_t k = 0; k < K; ++k) out[i * K + k] = double(t[k * npad + i]);
-    } else {
-        const double* t = reinterpret_cast<const double*>(tmp.data());
-        for (size_t i = 0; i < n; ++i)
-            for (size_t k = 0; k < K; ++k) out[i * K + k] = t[k * npad + i];
+    const ProbLayout& lay = h->lay;
+    size_t bytes = h->ops->elem() * size_t(lay.npad) * size_t(lay.K);
+    void* scratch = h->d_tmp;
+    Temps t(h->stream);
+    const size_t least = sizeof(double) * kRmRows * size_t(lay.K);
+    if (dev == h->d_tmp || bytes < least) {
+        bytes = std::max(least, std::min(2 * bytes, size_t(8) << 20));
+        FW_TRY(t.get(&scratch, bytes));
     }
-    return FW_OK;
+    return rowmajor_to_host(h->ops.get(), dev, lay.n, lay.npad, lay.K, out, scratch, bytes,
+                            h->stream);
 }
 
 // ---------------------------------------------------------------- profile
