@@ -15,6 +15,7 @@ constexpr int kResWarps = kResThreads / 32;
 constexpr int kResRing = 32;                      // iterations between statistics
 constexpr int kResTilesPerLayer = kResThreads / kBlock;   // row tiles per layer of a block
 constexpr int kResMaxCluster = 16;
+constexpr int kResMaxGrid = 160;                  // blocks of a grid group
 constexpr int kResMaxLen = 255;                   // chunks of 4 entries in the longest row
 constexpr int kResSmemMax = 220 * 1024;           // dynamic shared memory (227 KB less the static)
 
@@ -69,7 +70,7 @@ struct ResArgs {
     int32_t iters;           // iterations of this launch
     int32_t pad_;
     uint32_t* bar;           // grid group: arrivals, zero at launch
-    ResSlot* slots;          // grid group: [group][kNumR]
+    ResSlot* slots;          // grid group: [kNumR][group]
 };
 
 // The block's part of the problem.
@@ -772,7 +773,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
                 }
             } else {
                 const uint4* src = reinterpret_cast<const uint4*>(pd.cls4) + sp.first / 32;
-#pragma unroll 4
+#pragma unroll 8
                 for (int i = tid; i < sp.window / 32; i += kResThreads)
                     reinterpret_cast<uint4*>(tab)[i] = __ldcg(src + i);
             }
@@ -806,17 +807,30 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
             if constexpr (SHARED) {
                 const char* cp = col0;
                 const WT* vp = val0;
+                // the next chunk and its classes are loaded before one is added
                 auto walk = [&](T* my, int cnt) {
-#pragma unroll 2
-                    for (int i = 0; i < cnt; ++i) {
-                        Chunk<WT, WIDE, SHARED> B;
-                        uint32_t sc[4];
-                        B.load(cp, vp, 0);
-                        cp += 32 * kColBytes;
-                        vp += 128;
-                        B.gather(tb, sc);
-                        B.add(sc, my);
+                    if (cnt <= 0) return;
+                    Chunk<WT, WIDE, SHARED> A, B;
+                    uint32_t sa[4], sb[4];
+                    A.load(cp, vp, 0);
+                    A.gather(tb, sa);
+                    int i = 0;
+                    for (; i + 2 < cnt; i += 2) {
+                        B.load(cp, vp, i + 1);
+                        B.gather(tb, sb);
+                        A.add(sa, my);
+                        A.load(cp, vp, i + 2);
+                        A.gather(tb, sa);
+                        B.add(sb, my);
                     }
+                    if (i + 1 < cnt) {
+                        B.load(cp, vp, i + 1);
+                        B.gather(tb, sb);
+                    }
+                    A.add(sa, my);
+                    if (i + 1 < cnt) B.add(sb, my);
+                    cp += cnt * (32 * kColBytes);
+                    vp += cnt * 128;
                 };
                 if (s_rp.direct) {   // rows in place: the bins are the row's sums
                     for (int l = 0; l < layers; ++l) {
@@ -938,7 +952,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
                              make_uint4(uint32_t(lo), uint32_t(lo >> 32), uint32_t(hi),
                                         uint32_t(hi >> 32)));
             } else if (lane == 0) {
-                reinterpret_cast<ulonglong2*>(a.slots)[rank * kNumR + warp] = make_ulonglong2(lo, hi);
+                reinterpret_cast<ulonglong2*>(a.slots)[warp * a.group + rank] = make_ulonglong2(lo, hi);
             }
         }
         if (a.cluster) {
@@ -967,11 +981,19 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
             if (warp < kNumR) {
                 unsigned long long lo = 0ull, hi = 0ull;
                 bool bad = false;
-                for (int d = lane; d < a.group; d += 32) {
-                    const ulonglong2 v =
-                        __ldcg(reinterpret_cast<const ulonglong2*>(a.slots) + d * kNumR + warp);
-                    bad |= v.y == kResBad;
-                    add128(lo, hi, v.x, v.y);
+                // all loads first: one round trip to L2 for up to kResMaxGrid blocks
+                ulonglong2 v[kResMaxGrid / 32];
+#pragma unroll
+                for (int i = 0; i < kResMaxGrid / 32; ++i) {
+                    const int d = lane + 32 * i;
+                    v[i] = make_ulonglong2(0ull, 0ull);
+                    if (d < a.group)
+                        v[i] = __ldcg(reinterpret_cast<const ulonglong2*>(a.slots) + warp * a.group + d);
+                }
+#pragma unroll
+                for (int i = 0; i < kResMaxGrid / 32; ++i) {
+                    bad |= v[i].y == kResBad;
+                    add128(lo, hi, v[i].x, v[i].y);
                 }
                 bad = __any_sync(0xffffffffu, bad);
                 warp_sum128<16, 1>(lo, hi);
@@ -1150,6 +1172,7 @@ public:
         if (maxlen > kResMaxLen) return false;
         const int nt = pd.ntiles;
         const int pairs = (nt + kResTilesPerLayer - 1) / kResTilesPerLayer;
+        sms = std::min(sms, kResMaxGrid);
         auto cluster_of = [](int blocks) {
             int c = 1;
             while (c < blocks) c *= 2;

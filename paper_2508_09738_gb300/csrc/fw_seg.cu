@@ -174,8 +174,8 @@ static int graph_launches(int m) { return 2 * m + 1; }
 // Plan the resident kernel for the assembled problem and lay out its slices.
 // Without a plan, or without the memory for it, the solve runs the two-kernel
 // path.  The slices and the handle's other arrays stay within
-// fw_seg_footprint (create's temporaries are gone by now) plus 64 KB, less than
-// the granularity of the pool, so callers that admit by it need not know.
+// fw_seg_footprint (create's temporaries are gone by now) plus 1 MB, less than
+// the pool grows by, so callers that admit by it need not know.
 static fw_status plan_resident(fw_seg* h) {
     if (h->opts.class_table != FW_TABLE_AUTO) return FW_OK;   // the caller asks for a pass B form
     h->res.reset(make_res(h->opts.weight_dtype, h->lay.K));
@@ -189,7 +189,7 @@ static fw_status plan_resident(fw_seg* h) {
     const size_t used = problem_bytes(lay, te, h->ops->welem(), h->pd.comb) + sizeof(ProbState) +
                         te * size_t(lay.npad) * size_t(lay.K) + 5 * n + 8 * (n / kBlock + 1);
     if (used + res_bytes(p) >
-        fw_seg_footprint(lay.n, lay.nnz, lay.K, h->opts.weight_dtype) + 65536)
+        fw_seg_footprint(lay.n, lay.nnz, lay.K, h->opts.weight_dtype) + (size_t(1) << 20))
         return FW_OK;
     char* m = nullptr;
     if (h->alloc(&m, res_bytes(p)) != FW_OK) return FW_OK;
