@@ -120,6 +120,7 @@ struct Slot {
     size_t roff = SIZE_MAX, rbytes = 0;   // its arrays in the pool,
     void* rmem = nullptr;                 // or in the library's pool
     int rhead = 0, rqueued = 0;           // serving: launches in flight (ring entries)
+    uint64_t rturn = 0;                   // when the slot's last launch ended, or it joined
 };
 
 constexpr int kResStreams = 32;   // streams the resident launches of a batch spread over
@@ -177,8 +178,10 @@ public:
     std::vector<int> h_res;                      // live slots with a plan
     ProbState* h_rring = nullptr;                // pinned [slots][2] (serving)
     std::vector<cudaEvent_t> rring_ev;           // [slots][2]
+    uint64_t rturns = 0;
     bool res_outside = false;                    // slices may come from the library's pool
     int res_share = 0;                           // ResKern::plan
+    bool crowded = false;                        // serving: other requests wait or run
     long long budget = 0;
     cudaGraphExec_t graph = nullptr;
     int graph_iters = -1;
@@ -384,10 +387,8 @@ public:
         work_dirty = true;
         *out = s;
         if (plain_path && schedule == FW_SCHED_ITEMS) {
-            // small requests alone on their SMs, larger ones two layers a
-            // block so that several fit beside each other
-            res_share = lay.ntiles <= kResTilesPerLayer * kResMaxCluster ? 1 : 2;
-            if (lay.n >= shared_max_rows) res_share = 0;
+            // beside other requests few SMs, else as many as serve it best
+            res_share = crowded && lay.n < shared_max_rows ? 3 : 0;
             rc = plan_res(s);
             if (rc != FW_OK) remove(s);
         }
@@ -426,6 +427,7 @@ public:
         FW_CUDA(res_build(k, sl.rargs, p, side));
         sl.res = p;
         sl.rhead = sl.rqueued = 0;
+        sl.rturn = ++rturns;
         if (!rfork) {
             FW_CUDA(cudaEventCreateWithFlags(&rfork, cudaEventDisableTiming));
             for (int i = 0; i < kResStreams; ++i) {
@@ -685,15 +687,26 @@ public:
             }
         return FW_OK;
     }
-    // The states after the oldest launch of each (the newer ones keep running).
+    // Wait until some launch of the set has ended, and take the states of those
+    // that have: first the one queued longest ago, so the wait is short, then
+    // whichever others are ready.
     fw_status res_collect(const std::vector<int>& set) {
+        int oldest = -1;
+        for (int s : set)
+            if (oldest < 0 || slots[size_t(s)].rturn < slots[size_t(oldest)].rturn) oldest = s;
+        FW_CUDA(cudaEventSynchronize(rring_ev[2 * size_t(oldest) + size_t(slots[size_t(oldest)].rhead)]));
         for (int s : set) {
             Slot& sl = slots[size_t(s)];
-            const size_t i = 2 * size_t(s) + size_t(sl.rhead);
-            FW_CUDA(cudaEventSynchronize(rring_ev[i]));
-            h_state[s] = h_rring[i];
-            sl.rhead ^= 1;
-            --sl.rqueued;
+            while (sl.rqueued > 0) {
+                const size_t i = 2 * size_t(s) + size_t(sl.rhead);
+                const cudaError_t e = cudaEventQuery(rring_ev[i]);
+                if (e == cudaErrorNotReady) break;
+                FW_CUDA(e);
+                h_state[s] = h_rring[i];
+                sl.rhead ^= 1;
+                --sl.rqueued;
+                sl.rturn = ++rturns;
+            }
         }
         return FW_OK;
     }
@@ -1476,7 +1489,20 @@ void fw_srv::loop() {
             const HostGraph hg{rq->n, rq->rp.data(), rq->col.data(), rq->w.data(), rq->K,
                                rq->labels.data()};
             int slot = -1;
+            {
+                std::lock_guard<std::mutex> lk(mu);
+                e.crowded = info.resident > 0 || !queue.empty();
+            }
             const fw_status ra = e.add(hg, rq->opts, rq->lay, &slot);
+            // a resident request starts at once, while the next one is uploaded
+            if (ra == FW_OK && rc == FW_OK && !piped && (nlive == 0 || !res.empty()) &&
+                e.slots[size_t(slot)].res.group > 0 && rq->lay.n < kAloneRows) {
+                rc = e.res_queue({slot}, 4 * iters);
+                if (rc == FW_OK) {
+                    res.push_back(slot);
+                    ++nlive;
+                }
+            }
             std::lock_guard<std::mutex> lk(mu);
             if (ra != FW_OK) {
                 Result r;

@@ -45,8 +45,9 @@ public:
     virtual void spmm_hat(const ProbDesc& pd, void* out, cudaStream_t s) = 0;
     // classic FW gap partials per row block (fresh LUf)
     virtual void lmo_gap(const ProbDesc& pd, const void* LUf, double* part, cudaStream_t s) = 0;
-    // One-Shot Frank-Wolfe labels (Alg. 4) in one CSR pass
-    virtual void oneshot(const ProbDesc& pd, int32_t* labels, cudaStream_t s) = 0;
+    // One-Shot Frank-Wolfe labels (Alg. 4) of rows [first, last) in one CSR pass
+    virtual void oneshot(const ProbDesc& pd, int32_t* labels, int first, int last,
+                         cudaStream_t s) = 0;
     virtual void build(int64_t n, const int32_t* rp, const int32_t* col, const double* w,
                        const double* deg, const int32_t* rpp, int32_t* colp, void* valp,
                        void* diag, int comb, int col16, cudaStream_t s) = 0;

@@ -422,13 +422,78 @@ static __global__ void k_finish(ProbDesc pd, ProbState* st) {   // one warp
 // CSR pass; the iterate arrays are not touched.  There is no reduction, so
 // each block takes one 256-row sub-tile (fine-grained, no tail wave).
 template <typename T, typename WT, int KMAX>
-__global__ void __launch_bounds__(kBlock) k_osfw(ProbDesc pd, int32_t* labels) {
+__global__ void __launch_bounds__(kBlock) k_osfw(ProbDesc pd, int32_t* labels, int first, int last) {
     extern __shared__ __align__(128) unsigned char smraw[];
     T* sm_lane = reinterpret_cast<T*>(smraw);
     T* sm_row = sm_lane + kBlock * (KMAX | 1);
-    const int r0 = blockIdx.x * kBlock;
-    const int r1 = min(pd.n, r0 + kBlock);
+    const int r0 = first + blockIdx.x * kBlock;
+    const int r1 = min(last, r0 + kBlock);
     osfw_rows<T, WT, KMAX>(pd, labels, r0, r1, sm_lane, sm_row);
+}
+
+// The same for a pattern problem with exactly K <= 8 classes (see
+// k_passB_pat): no row offsets or columns are read, and the sums stay in
+// registers.  A labelled neighbour of class c adds fma(v, 1, .) to c and
+// fma(v, 0, .) to the others, an unlabelled one fma(v, 1/K, .) to every class:
+// the sums of csr_bins, branch-free.  Bound by its 37 bytes a row (FP32) from
+// HBM and its instructions; the general kernel took 91 us on the 2048 x 2048
+// image (K = 4), issue-bound on columns, bins and guards.
+template <typename WT, int K>
+__global__ void __launch_bounds__(kBlock) k_osfw_pat(ProbDesc pd, int32_t* labels, int first,
+                                                     int last) {
+    __shared__ __align__(16) int16_t s_tab[kPatterns][kPatRow];
+    if (threadIdx.x < kPatterns * kPatRow / 8)
+        reinterpret_cast<uint4*>(s_tab)[threadIdx.x] =
+            __ldg(reinterpret_cast<const uint4*>(pd.ptab) + threadIdx.x);
+    const int r = first + blockIdx.x * kBlock + threadIdx.x;
+    const bool in = r < last;
+    float w[kPatRow];
+    int pid = 0, f = -1;
+    if (in) {
+        pid = __ldg(pd.pat + r);
+        f = __ldg(pd.fid + r);
+        ld_w8(static_cast<const WT*>(pd.val) + int64_t(r) * kPatRow, w);
+    }
+    __syncthreads();
+    if (!in) return;
+    const uint4 o4 = *reinterpret_cast<const uint4*>(s_tab[pid]);
+    const uint32_t ow[4] = {o4.x, o4.y, o4.z, o4.w};
+    int fj[kPatRow];
+#pragma unroll
+    for (int i = 0; i < kPatRow; ++i) {
+        const int off = i & 1 ? int(ow[i / 2]) >> 16 : int(ow[i / 2] << 16) >> 16;
+        fj[i] = __ldg(pd.fid + uint32_t(r + off));
+    }
+    const float unif = 1.f / float(K);
+    float b[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) b[k] = 0.f;
+#pragma unroll
+    for (int i = 0; i < kPatRow; ++i) {
+        const float other = fj[i] < 0 ? unif : 0.f;
+#pragma unroll
+        for (int k = 0; k < K; ++k) b[k] = fma_(w[i], fj[i] == k ? 1.f : other, b[k]);
+    }
+    const float c2 = pd.c2f, om = pd.omf;
+    const bool greedy = pd.oracle == 0;
+    const float dg = pd.comb ? static_cast<const float*>(pd.diag)[r] : 1.f;
+    int s = f;   // a labelled row is binary: the greedy rule keeps its class
+    if (f < 0 || !greedy) {
+        float best = CUDART_INF_F;
+        s = -1;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const float u = uhat_val<float>(f, k, unif);
+            float gk = fma_(-c2, u, sub_(mul_(dg, u), b[k]));
+            if (f >= 0) gk = fma_(om, sub_(u, k == f ? 1.f : 0.f), gk);
+            if (gk < best) {   // unlabelled rows admit every class, the full LMO too
+                best = gk;
+                s = k;
+            }
+        }
+        if (s < 0) s = 0;
+    }
+    labels[r] = s;
 }
 
 // OUT = L X (initial L U_0, refresh, direct objective).

@@ -171,8 +171,23 @@ public:
     void finish(const ProbDesc& pd, ProbState* st, cudaStream_t s) override {
         k_finish<<<1, 32, 0, s>>>(pd, st);
     }
-    void oneshot(const ProbDesc& pd, int32_t* labels, cudaStream_t s) override {
-        k_osfw<T, WT, KMAX><<<rows_grid(pd), kBlock, smem(), s>>>(pd, labels);
+    void oneshot(const ProbDesc& pd, int32_t* labels, int first, int last,
+                 cudaStream_t s) override {
+        const unsigned g = unsigned((last - first + kBlock - 1) / kBlock);
+        if constexpr (kPat) {
+            if (pd.pat) {
+                switch (pd.K) {
+                    case 2: if constexpr (KMAX == 4) k_osfw_pat<WT, 2><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
+                    case 3: if constexpr (KMAX == 4) k_osfw_pat<WT, 3><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
+                    case 4: if constexpr (KMAX == 4) k_osfw_pat<WT, 4><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
+                    case 5: if constexpr (KMAX == 8) k_osfw_pat<WT, 5><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
+                    case 6: if constexpr (KMAX == 8) k_osfw_pat<WT, 6><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
+                    case 7: if constexpr (KMAX == 8) k_osfw_pat<WT, 7><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
+                    default: if constexpr (KMAX == 8) k_osfw_pat<WT, 8><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
+                }
+            }
+        }
+        k_osfw<T, WT, KMAX><<<g, kBlock, smem(), s>>>(pd, labels, first, last);
     }
     void spmm_hat(const ProbDesc& pd, void* out, cudaStream_t s) override {
         k_spmm_hat<T, WT, KMAX><<<pd.ntiles, kBlock, smem(), s>>>(pd, (T*)out);

@@ -45,6 +45,8 @@ static fw_status invalid(const std::string& m) {
         if (s_ != FW_OK) return s_;        \
     } while (0)
 
+constexpr int kCopyParts = 2;
+
 struct fw_seg {
     int device = 0;
     fw_seg_opts opts{};
@@ -66,9 +68,12 @@ struct fw_seg {
     std::unique_ptr<ResKern> res;      // solves run resident when res_plan.group > 0
     ResPlan res_plan;
     ResArgs res_args{};                // its launch parameters but the iteration count
+    bool pat_tried = false;            // plan_patterns has run
     int last_refresh = 0;
     int launches = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    cudaStream_t copy_stream = nullptr;            // label parts of fw_seg_oneshot
+    cudaEvent_t part_ev[kCopyParts] = {};
     std::vector<void*> dev_allocs;
 
     // device arrays: stream-ordered on the handle's stream, from the
@@ -88,6 +93,12 @@ struct fw_seg {
         for (void* p : dev_allocs) cudaFreeAsync(p, stream);   // back to the pool
         if (h_state) cudaFreeHost(h_state);   // h_ring lives in the same block
         for (cudaEvent_t e : ring_ev)
+            if (e) cudaEventDestroy(e);
+        if (copy_stream) {
+            cudaStreamSynchronize(copy_stream);
+            cudaStreamDestroy(copy_stream);
+        }
+        for (cudaEvent_t e : part_ev)
             if (e) cudaEventDestroy(e);
         if (ev0) cudaEventDestroy(ev0);
         if (ev1) cudaEventDestroy(ev1);
@@ -199,12 +210,14 @@ static fw_status plan_resident(fw_seg* h) {
     return FW_OK;
 }
 
-// Find the offset patterns of a regular grid, for the pass B that reads no
-// columns.  Not for problems the resident kernel takes, nor when the caller
-// asks for a pass B form.
+// Find the offset patterns of a regular grid, for the pass B and the one-shot
+// pass that read no columns; not when the caller asks for a pass B form.  At
+// create, or, where the resident kernel takes the solves, at the first
+// one-shot call.
 static fw_status plan_patterns(fw_seg* h) {
     const ProbLayout& lay = h->lay;
-    if (h->res_plan.group > 0 || h->opts.class_table != FW_TABLE_AUTO || h->pd.tab_grid > 0 ||
+    h->pat_tried = true;
+    if (h->opts.class_table != FW_TABLE_AUTO || h->pd.tab_grid > 0 ||
         lay.padw != kPatRow || !h->pd.col16 || h->pd.lanes != 1 ||
         !h->ops->pattern_kernels(lay.K))
         return FW_OK;
@@ -468,7 +481,7 @@ fw_status fw_seg_create(fw_seg** out, int64_t n, const int32_t* row_ptr, const i
         FW_TRY(assemble_uploaded(h->ops.get(), *up, lay, h->pd, h->st, h->stream));
         up.reset();   // its device copies go back to the pool
         FW_TRY(plan_resident(h.get()));
-        FW_TRY(plan_patterns(h.get()));
+        if (h->res_plan.group == 0) FW_TRY(plan_patterns(h.get()));
         FW_TRY(read_state(h.get()));
         if (h->res_plan.group == 0 && build_graph(h.get()) != FW_OK) {
             // streams that cannot be captured (the legacy default stream) run
@@ -674,14 +687,42 @@ fw_status fw_seg_labels(fw_seg* h, int32_t* labels_host) {
 
 fw_status fw_seg_oneshot(fw_seg* h, int32_t* labels_host, double* ms) {
     if (!h) return invalid("handle is NULL");
-    FW_CUDA(cudaEventRecord(h->ev0, h->stream));
-    h->ops->oneshot(h->pd, h->d_labels, h->stream);
-    FW_TRY(launch_check("one-shot kernel"));
-    FW_CUDA(cudaEventRecord(h->ev1, h->stream));
-    if (labels_host)
-        FW_CUDA(cudaMemcpyAsync(labels_host, h->d_labels, 4 * size_t(h->lay.n),
-                                cudaMemcpyDeviceToHost, h->stream));
-    FW_CUDA(cudaStreamSynchronize(h->stream));
+    if (!h->pat_tried) FW_TRY(plan_patterns(h));
+    // Large label arrays leave in parts, each copied (on a stream of the
+    // handle's own, behind the part's kernel) while the next part is computed:
+    // at 2048 x 2048 the copy takes 89 us, the kernel a third of that.
+    const int n = h->pd.n;
+    const int parts = labels_host && n >= (1 << 20) ? kCopyParts : 1;
+    if (parts > 1 && !h->copy_stream) {
+        FW_CUDA(cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking));
+        for (cudaEvent_t& e : h->part_ev)
+            FW_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    }
+    auto cut = [n, parts](int i) { return int(int64_t(n) * i / parts) & ~(kBlock - 1); };
+    auto enqueue = [&]() -> cudaError_t {
+        cudaError_t e = cudaEventRecord(h->ev0, h->stream);
+        for (int i = 0; i < parts && e == cudaSuccess; ++i) {
+            h->ops->oneshot(h->pd, h->d_labels, cut(i), i + 1 < parts ? cut(i + 1) : n, h->stream);
+            e = cudaGetLastError();
+            if (e == cudaSuccess && parts > 1) e = cudaEventRecord(h->part_ev[i], h->stream);
+        }
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev1, h->stream);
+        for (int i = 0; i < parts && labels_host && e == cudaSuccess; ++i) {
+            const cudaStream_t s = parts > 1 ? h->copy_stream : h->stream;
+            const int r0 = cut(i), r1 = i + 1 < parts ? cut(i + 1) : n;
+            if (parts > 1) e = cudaStreamWaitEvent(s, h->part_ev[i], 0);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(labels_host + r0, h->d_labels + r0, 4 * size_t(r1 - r0),
+                                    cudaMemcpyDeviceToHost, s);
+        }
+        return e;
+    };
+    const cudaError_t e0 = enqueue();
+    // also after an error: nothing writes the caller's array after the return
+    const cudaError_t e1 = parts > 1 ? cudaStreamSynchronize(h->copy_stream) : cudaSuccess;
+    const cudaError_t e2 = cudaStreamSynchronize(h->stream);
+    for (cudaError_t e : {e0, e1, e2})
+        if (e != cudaSuccess) return cuda_fail(e, "one-shot pass");
     if (ms) {
         float t = 0.f;
         FW_CUDA(cudaEventElapsedTime(&t, h->ev0, h->ev1));

@@ -110,3 +110,31 @@ def test_solves_in_parts():
         sa, sb = a.solve(), b.solve()
         assert (sa.iters, sa.gap, sa.objective) == (sb.iters, sb.gap, sb.objective)
         assert np.array_equal(a.U(), b.U())
+
+
+# regular grids past the resident kernel: pass B and the one-shot pass from row
+# patterns, against the column-reading forms (32-bit indices never use patterns)
+@pytest.mark.parametrize("weights", ["f32", "bf16"])
+@pytest.mark.parametrize("side,height,K,opts", [
+    (601, 520, 4, {}), (601, 520, 2, dict(laplacian="comb")), (1031, 977, 3, {}),
+    (640, 500, 8, dict(oracle="full")), (640, 500, 5, dict(eps=0.1)), (320, 1000, 7, {}),
+    (2400, 2101, 6, {})])
+def test_patterns_equal_columns(weights, side, height, K, opts):
+    g = W.voronoi_image(side=side, height=height, K=K, label_frac=0.01, seed=side + K)
+    kw = dict(weight_dtype=weights, max_iters=12, omega0=1e5, **opts)
+    with B.Segmenter(g, **kw) as a, B.Segmenter(g, index_width=32, **kw) as b:
+        assert a.forms().index_width == 16 and b.forms().index_width == 32
+        assert np.array_equal(a.oneshot()[0], b.oneshot()[0])
+        sa, sb = a.solve(), b.solve()
+        for f in STATS:
+            assert getattr(sa, f) == getattr(sb, f), f
+        assert np.array_equal(a.U(), b.U())
+        assert np.array_equal(a.labels(), b.labels())
+
+
+def test_oneshot_patterns_on_a_resident_problem():
+    g = W.voronoi_image(side=211, height=90, K=5, label_frac=0.02, seed=2)
+    with B.Segmenter(g, eps=0.1, omega0=1e5) as a, \
+            B.Segmenter(g, eps=0.1, omega0=1e5, index_width=32) as b:
+        assert np.array_equal(a.oneshot()[0], b.oneshot()[0])
+        assert a.solve().gap == b.solve().gap
