@@ -796,7 +796,7 @@ __device__ __forceinline__ int warp_finish(const ProbDesc& pd, ProbState* st,
 
 // Staged pass A over rows [r_begin, r_end) in 256-row sub-tiles.  For each
 // sub-tile one thread issues bulk copies of its class columns of U, LU (and LS
-// when a step is pending) into a stage buffer (T[3][KMAX][256]) completing on
+// when a step is pending) into a stage buffer (T[3][K][256]) completing on
 // that buffer's mbarrier; with two stages the copies of sub-tile j+1 are in
 // flight while sub-tile j is computed.  Each thread updates and evaluates its
 // row from shared memory in two sweeps (argmin, then the gap terms), with the
@@ -825,8 +825,8 @@ __device__ __forceinline__ void stage_issue(const ProbDesc& pd, int base, int ro
     const T* LSb = static_cast<const T*>(pd.LS);
     for (int k = 0; k < K; ++k) {
         bulk_g2s(stage + k * kBlock, Ub + k * np + base, seg, bar);
-        bulk_g2s(stage + (KMAX + k) * kBlock, LUb + k * np + base, seg, bar);
-        if (upd) bulk_g2s(stage + (2 * KMAX + k) * kBlock, LSb + k * np + base, seg, bar);
+        bulk_g2s(stage + (K + k) * kBlock, LUb + k * np + base, seg, bar);
+        if (upd) bulk_g2s(stage + (2 * K + k) * kBlock, LSb + k * np + base, seg, bar);
     }
 }
 
@@ -860,7 +860,7 @@ __device__ __forceinline__ int passA_staged(const ProbDesc& pd, int r_begin, int
     T oma = sub_(T(1), alpha);
     const bool greedy = pd.oracle == 0;
     const T floor_u = greedy ? T(0) : -inf_<T>();   // admissible classes: u > floor_u
-    const int stage_elems = 3 * KMAX * kBlock;
+    const int stage_elems = 3 * K * kBlock;
     int rc = kPassOk;
     // with fc.fin the caller has issued the first sub-tile's copies and taken
     // the decision (s_stop, s_alpha) before calling
@@ -875,8 +875,8 @@ __device__ __forceinline__ int passA_staged(const ProbDesc& pd, int r_begin, int
             stage_issue<T, KMAX>(pd, base, min(kBlock, r_end - base), upd, stage, &bars[0]);
         const int rows = min(kBlock, r_end - base);
         T* sU = stage + buf * stage_elems;
-        T* sL = sU + KMAX * kBlock;
-        T* sS = sU + 2 * KMAX * kBlock;
+        T* sL = sU + K * kBlock;
+        T* sS = sU + 2 * K * kBlock;
         const int t = threadIdx.x;
         const int r = base + t;
         // per-row bytes are loaded before the wait so their latency overlaps the copies

@@ -151,14 +151,20 @@ __global__ void __launch_bounds__(kBlock, MODE == MODE_STEP ? passA_min_blocks<T
     }
 }
 
-// Pass A (step) for exactly KMAX classes with an FP32 iterate: the class loop
-// is fully known at compile time, which removes the per-class guards.  Used
-// for four classes, where it is held to 32 registers (8 blocks per SM).
-template <typename T, int KMAX>
-__global__ void __launch_bounds__(kBlock, passA_min_blocks<T, KMAX>())
+// Pass A (step) for exactly K <= 8 classes with an FP32 iterate: the class loop
+// is fully known at compile time, which removes the per-class guards, and the
+// registers are bounded by the blocks whose two stage buffers (of K classes,
+// not of the class bound) one SM holds.
+template <int K>
+constexpr int passA_exact_blocks() {
+    constexpr int b = (227 * 1024) / (2 * 3 * kBlock * K * 4 + 1024);
+    return b > 8 ? 8 : b;
+}
+template <typename T, int K>
+__global__ void __launch_bounds__(kBlock, passA_exact_blocks<K>())
     k_passA_exact(ProbDesc pd, ProbState* st, int fin) {
     extern __shared__ __align__(128) unsigned char smraw[];
-    passA_step<T, KMAX, true>(pd, st, fin, reinterpret_cast<T*>(smraw), blockIdx.x);
+    passA_step<T, K, true>(pd, st, fin, reinterpret_cast<T*>(smraw), blockIdx.x);
 }
 
 // Pass B: one block per row tile; each adds its tile total to the exact

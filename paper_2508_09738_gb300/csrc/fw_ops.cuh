@@ -8,10 +8,9 @@ namespace fw {
 template <typename T, typename WT, int KMAX>
 class OpsImpl final : public Ops {
 public:
-    // exactly KMAX classes, FP32 iterate: the compile-time class-count forms
-    // (pass A only for four classes: with more, the fully unrolled row keeps
-    // its classes in registers and spills at the occupancy it needs)
-    static constexpr bool kExactA = sizeof(T) == 4 && KMAX == 4;
+    // FP32 iterate: the compile-time class-count forms (pass A for each K of
+    // at most 8 classes, pass B where K is the class bound)
+    static constexpr bool kExactA = sizeof(T) == 4 && KMAX <= 8;
     static constexpr bool kExactB = sizeof(T) == 4 && KMAX <= 12;
     // 2 / 4 lanes per row, 5..12 classes, FP32 iterate: the 40-register pass B
     static constexpr bool kBound6 = sizeof(T) == 4 && KMAX >= 8 && KMAX <= 12;
@@ -33,8 +32,25 @@ public:
     }
     static size_t smemA() { return max_stages<T, KMAX>() * 3 * size_t(kBlock) * KMAX * sizeof(T); }
     static size_t smemA(const ProbDesc& pd) {
-        return (pd.tile_rows > kBlock ? max_stages<T, KMAX>() : 1) * 3 * size_t(kBlock) * KMAX *
-               sizeof(T);
+        return (pd.tile_rows > kBlock ? max_stages<T, KMAX>() : 1) * 3 * size_t(kBlock) *
+               size_t(pd.K) * sizeof(T);
+    }
+    // f(the exact pass A of K classes), for K this class bound serves
+    template <typename F>
+    static cudaError_t exactA(int K, F f) {
+        if constexpr (kExactA) {
+            switch (K) {
+                case 2: if constexpr (KMAX == 4) return f(k_passA_exact<T, 2>); break;
+                case 3: if constexpr (KMAX == 4) return f(k_passA_exact<T, 3>); break;
+                case 4: if constexpr (KMAX == 4) return f(k_passA_exact<T, 4>); break;
+                case 5: if constexpr (KMAX == 8) return f(k_passA_exact<T, 5>); break;
+                case 6: if constexpr (KMAX == 8) return f(k_passA_exact<T, 6>); break;
+                case 7: if constexpr (KMAX == 8) return f(k_passA_exact<T, 7>); break;
+                case 8: if constexpr (KMAX == 8) return f(k_passA_exact<T, 8>); break;
+                default: break;
+            }
+        }
+        return cudaErrorInvalidValue;
     }
     static unsigned rows_grid(const ProbDesc& pd) { return unsigned((pd.n + kBlock - 1) / kBlock); }
 
@@ -43,11 +59,14 @@ public:
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              int(smemA()));
         if (e != cudaSuccess) return e;
-        if constexpr (kExactA) {
-            e = cudaFuncSetAttribute(k_passA_exact<T, KMAX>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, int(smemA()));
-            if (e != cudaSuccess) return e;
-        }
+        if constexpr (kExactA)
+            for (int K = KMAX / 2 + (KMAX == 8); K <= KMAX; ++K) {
+                e = exactA(K, [](auto kern) {
+                    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                int(smemA()));
+                });
+                if (e != cudaSuccess) return e;
+            }
         e = cudaFuncSetAttribute(k_passB<T, WT, KMAX>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(smemB()));
         if (e != cudaSuccess) return e;
@@ -87,10 +106,11 @@ public:
     void passA(const ProbDesc& pd, ProbState* st, cudaStream_t s, int fin) override {
         const unsigned grid = unsigned(pd.ntiles) + (fin ? 1u : 0u);   // see passA_step
         if constexpr (kExactA) {
-            if (pd.K == KMAX) {
-                k_passA_exact<T, KMAX><<<grid, kBlock, smemA(pd), s>>>(pd, st, fin);
-                return;
-            }
+            exactA(pd.K, [&](auto kern) {
+                kern<<<grid, kBlock, smemA(pd), s>>>(pd, st, fin);
+                return cudaSuccess;
+            });
+            return;
         }
         k_passA<T, KMAX, MODE_STEP><<<grid, kBlock, smemA(pd), s>>>(pd, st, nullptr, nullptr, fin);
     }
