@@ -344,7 +344,9 @@ typedef struct fw_batch fw_batch;
  * or 16).  The schedule, the class bound and the launch length change no
  * result; the lanes per row change the order in which a row's entries are
  * summed, so a batch equals single solves bit for bit when those use the
- * same lanes_per_row (fw_batch_info reports it).  The choice is cached in
+ * same lanes_per_row (fw_batch_info reports it).  When the resident kernel
+ * takes every problem, nothing is timed: per-item schedule, each problem's own
+ * lanes, all iterations in one launch.  The choice is cached in
  * tune_cache under a signature of the device and the batch's sizes. */
 fw_status fw_batch_default_opts(fw_batch_opts *opts);
 

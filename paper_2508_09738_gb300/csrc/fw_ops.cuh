@@ -55,11 +55,12 @@ public:
     static unsigned rows_grid(const ProbDesc& pd) { return unsigned((pd.n + kBlock - 1) / kBlock); }
 
     cudaError_t configure() override {
-        cudaError_t e = cudaFuncSetAttribute(k_passA<T, KMAX, MODE_STEP>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(smemA()));
-        if (e != cudaSuccess) return e;
-        if constexpr (kExactA)
+        cudaError_t e = cudaSuccess;
+        if constexpr (!kExactA) {
+            e = cudaFuncSetAttribute(k_passA<T, KMAX, MODE_STEP>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, int(smemA()));
+            if (e != cudaSuccess) return e;
+        } else {
             for (int K = KMAX / 2 + (KMAX == 8); K <= KMAX; ++K) {
                 e = exactA(K, [](auto kern) {
                     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -67,6 +68,7 @@ public:
                 });
                 if (e != cudaSuccess) return e;
             }
+        }
         e = cudaFuncSetAttribute(k_passB<T, WT, KMAX>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(smemB()));
         if (e != cudaSuccess) return e;
@@ -110,9 +112,10 @@ public:
                 kern<<<grid, kBlock, smemA(pd), s>>>(pd, st, fin);
                 return cudaSuccess;
             });
-            return;
+        } else {
+            k_passA<T, KMAX, MODE_STEP><<<grid, kBlock, smemA(pd), s>>>(pd, st, nullptr, nullptr,
+                                                                         fin);
         }
-        k_passA<T, KMAX, MODE_STEP><<<grid, kBlock, smemA(pd), s>>>(pd, st, nullptr, nullptr, fin);
     }
     void flush(const ProbDesc& pd, ProbState* st, cudaStream_t s) override {
         k_passA<T, KMAX, MODE_FLUSH><<<pd.ntiles, kBlock, 0, s>>>(pd, st, nullptr, nullptr, 0);

@@ -487,9 +487,9 @@ __device__ __forceinline__ unsigned long long ring_word(const ResSlot* tot, int 
 // tenth cycle, four warps a scheduler), for small problems the exchange, the
 // longest row of the graph and the one-warp decision; registers (two values
 // per row and class) allow no more warps.  Two launches an iteration took
-// 14.3 us where this takes 4.8 (2,000-point k-NN graph, K = 5), 14.4 -> 8.5
-// (22,470 points, K = 7), 24.0 -> 11.9 (613 x 487 image, K = 6) and 31.8 ->
-// 22.2 (200,000-node block model, K = 10: the walk waits on L2 there).
+// 14.3 us where this takes 4.7 (2,000-point k-NN graph, K = 5), 14.4 -> 8.4
+// (22,470 points, K = 7), 24.0 -> 10.6 (613 x 487 image, K = 6) and 31.8 ->
+// 21.4 (200,000-node block model, K = 10: the walk waits on L2 there).
 //
 // FORM kResWide: 4-bit class table and 32-bit columns; else one byte per row
 // and 16-bit columns (a table of at most 65,536 rows), with kResShared the

@@ -68,7 +68,6 @@ struct fw_seg {
     std::unique_ptr<ResKern> res;      // solves run resident when res_plan.group > 0
     ResPlan res_plan;
     ResArgs res_args{};                // its launch parameters but the iteration count
-    bool pat_tried = false;            // plan_patterns has run
     int last_refresh = 0;
     int launches = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -212,11 +211,11 @@ static fw_status plan_resident(fw_seg* h) {
 
 // Find the offset patterns of a regular grid, for the pass B and the one-shot
 // pass that read no columns; not when the caller asks for a pass B form.  At
-// create, or, where the resident kernel takes the solves, at the first
-// one-shot call.
+// create, and not where the resident kernel takes the solves: there only the
+// one-shot pass would use them, and finding them at its first call took 42 us
+// (107 us against 65) where later calls gained 1 of 32.
 static fw_status plan_patterns(fw_seg* h) {
     const ProbLayout& lay = h->lay;
-    h->pat_tried = true;
     if (h->opts.class_table != FW_TABLE_AUTO || h->pd.tab_grid > 0 ||
         lay.padw != kPatRow || !h->pd.col16 || h->pd.lanes != 1 ||
         !h->ops->pattern_kernels(lay.K))
@@ -687,10 +686,10 @@ fw_status fw_seg_labels(fw_seg* h, int32_t* labels_host) {
 
 fw_status fw_seg_oneshot(fw_seg* h, int32_t* labels_host, double* ms) {
     if (!h) return invalid("handle is NULL");
-    if (!h->pat_tried) FW_TRY(plan_patterns(h));
     // Large label arrays leave in parts, each copied (on a stream of the
     // handle's own, behind the part's kernel) while the next part is computed:
-    // at 2048 x 2048 the copy takes 89 us, the kernel a third of that.
+    // at 2048 x 2048 the copy takes 89 us, the kernel about 50 in two parts,
+    // the call 145 instead of 205 (four parts: 10 more).
     const int n = h->pd.n;
     const int parts = labels_host && n >= (1 << 20) ? kCopyParts : 1;
     if (parts > 1 && !h->copy_stream) {

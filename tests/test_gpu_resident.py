@@ -132,7 +132,7 @@ def test_patterns_equal_columns(weights, side, height, K, opts):
         assert np.array_equal(a.labels(), b.labels())
 
 
-def test_oneshot_patterns_on_a_resident_problem():
+def test_oneshot_on_a_resident_problem():
     g = W.voronoi_image(side=211, height=90, K=5, label_frac=0.02, seed=2)
     with B.Segmenter(g, eps=0.1, omega0=1e5) as a, \
             B.Segmenter(g, eps=0.1, omega0=1e5, index_width=32) as b:
