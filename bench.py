@@ -128,22 +128,42 @@ def column_bytes(g) -> int:
     return 4 if far else 2
 
 
-def bytes_per_unit(n, nnz, K, wbytes, tbytes=4, cbytes=4):
+def reads_patterns(g, forms, tbytes=4, class_table="auto") -> bool:
+    """Whether pass B and the one-shot pass take one pattern byte per row in
+    place of row offsets and columns: regular grids with at most 64 distinct
+    rows of 5 to 8 entries, K <= 8, an FP32 iterate, one lane per row, and more
+    rows than the resident kernel takes (mirrors the library's rule)."""
+    d = np.diff(g.row_ptr).astype(np.int64)
+    if (not forms or class_table != "auto" or tbytes != 4 or g.K > 8 or g.n <= 311_296
+            or forms.get("class_table") or forms.get("lanes_per_row") != 1
+            or forms.get("index_width") != 16 or not 4 < d.max() <= 8 or g.nnz < 5 * g.n
+            or 8 * g.n > 1.02 * ((d + 3) // 4 * 4).sum()):
+        return False
+    rows = np.repeat(np.arange(g.n, dtype=np.int64), d)
+    at = np.arange(g.nnz, dtype=np.int64) - np.repeat(g.row_ptr[:-1].astype(np.int64), d)
+    off = np.zeros((g.n, 8), dtype=np.int16)
+    off[rows, at] = g.col.astype(np.int64) - rows
+    return len(np.unique(off.view("V16").ravel())) <= 64
+
+
+def bytes_per_unit(n, nnz, K, wbytes, tbytes=4, cbytes=4, patterns=False):
     """Algorithmic bytes of one FW iteration (the method's minimum: U and L U
     read and written, the CSR once, row_ptr, choice and fidelity bytes) and of
     each pass of the two-pass design (pass A: U, L U, L S in, U, L U out;
     pass B: U in for the moved rows, L S out, the CSR, row_ptr, the row's own
-    choice and the gathered neighbour classes)."""
+    choice and the gathered neighbour classes; with row patterns one byte a row
+    in place of columns and row_ptr)."""
     row_pass = 5 * tbytes * n * K + 3 * n                 # U, LU, LS in; U, LU out; choice, fid
-    csr_pass = (2 * tbytes * n * K + (cbytes + wbytes) * nnz   # U in, LS out; col + weights
-                + 4 * (n + 1) + 2 * n)                    # row_ptr; choice of the row + gathers
+    index = n if patterns else cbytes * nnz + 4 * (n + 1)
+    csr_pass = (2 * tbytes * n * K + wbytes * nnz         # U in, LS out; weights
+                + index + 2 * n)                          # columns; choice of the row + gathers
     iteration = 4 * tbytes * n * K + (4 + wbytes) * nnz + 4 * n + 3 * n
     return dict(row_pass=row_pass, csr_pass=csr_pass, iteration=iteration)
 
 
 # the sources that define and instantiate the profiled kernels (pass A,
 # pass B, finish, one-shot); host-only set-up and driver code is not included
-KERNEL_SOURCES = ("fw_types.h", "fw_device.cuh", "fw_kernels.cuh", "fw_ops.cuh",
+KERNEL_SOURCES = ("fw_types.h", "fw_step.cuh", "fw_device.cuh", "fw_kernels.cuh", "fw_ops.cuh",
                   "fw_ops_f32.cu", "fw_ops_bf16.cu", "fw_ops_f64.cu")
 
 
@@ -633,9 +653,11 @@ def run_oneshot(args, rank, world, local):
         st = seg.solve()
         gfw_ms.append(st.ms)
     lab_gfw = seg.labels()
+    pat = reads_patterns(g, seg.forms().as_dict(), 8 if weights == "f64" else 4)
     seg.close()
     wb = {"f32": 4, "bf16": 2, "f64": 8}[weights]
-    nbytes = 4 * (g.n + 1) + (column_bytes(g) + wb) * g.nnz + g.n + 4 * g.n
+    index = g.n if pat else 4 * (g.n + 1) + column_bytes(g) * g.nnz
+    nbytes = index + wb * g.nnz + g.n + 4 * g.n
     mean_ms = float(np.mean(kms))
     peaks = load_peaks()
     achieved = nbytes / (mean_ms / 1000.0) / 1e9
@@ -758,10 +780,11 @@ def compare_golden(gold, labels, E_gpu, traj, truth):
     return d
 
 
-def roofline_of(prof, g, weights, workload, peaks, forms=None):
+def roofline_of(prof, g, weights, workload, peaks, forms=None, class_table="auto"):
     wb = {"f32": 4, "bf16": 2, "f64": 8}[weights]
     tb = 8 if weights == "f64" else 4
-    by = bytes_per_unit(g.n, g.nnz, g.K, wb, tb, column_bytes(g))
+    pat = reads_patterns(g, forms, tb, class_table)
+    by = bytes_per_unit(g.n, g.nnz, g.K, wb, tb, column_bytes(g), pat)
     dom = "csr_pass" if prof["pass_b"] >= prof["pass_a"] else "row_pass"
     dom_ms = prof["pass_b"] if dom == "csr_pass" else prof["pass_a"]
     kernel = {"csr_pass": "k_passB", "row_pass": "k_passA"}[dom]
@@ -771,7 +794,8 @@ def roofline_of(prof, g, weights, workload, peaks, forms=None):
             "frac": achieved / peaks["hbm_gbs"], "traffic": ncu_traffic(kernel, key),
             "kernel": kernel, "peak_source": peaks["source"],
             "kernel_form": (("k_passB_tab (class table in shared memory)"
-                             if forms and forms.get("class_table") else "k_passB_lc / k_passB")
+                             if forms and forms.get("class_table") else
+                             "k_passB_pat (row patterns)" if pat else "k_passB_lc / k_passB")
                             if kernel == "k_passB" else "k_passA"),
             "algorithmic_bytes_per_launch": by[dom],
             "timing": "CUDA events on the solver's stream around a captured graph of "
@@ -827,7 +851,8 @@ def time_arm(args, B, torch, g, c, weights, iters, stream, flush, clocks, world,
 
 def arm_record(args, arm, g, c, weights, iters, world, peaks):
     """The JSON fields of one timed weight dtype."""
-    roof, by = roofline_of(arm["prof"], g, weights, args.workload, peaks, arm.get("forms"))
+    roof, by = roofline_of(arm["prof"], g, weights, args.workload, peaks, arm.get("forms"),
+                           args.class_table)
     ms_step = 1000.0 * arm["t_s"] / args.steps
     rec = {"value": arm["value"], "unit": "iter/s", "weights": weights,
            "ms_per_step": ms_step, "solves_per_s": world * args.steps / arm["t_s"],
