@@ -425,15 +425,22 @@ public:
         sl.rbytes = need;
         sl.rk = k;
         FW_CUDA(res_build(k, sl.rargs, p, side));
+        FW_TRY(res_streams(std::min(s + 1, kResStreams)));
         sl.res = p;
         sl.rhead = sl.rqueued = 0;
         sl.rturn = ++rturns;
-        if (!rfork) {
-            FW_CUDA(cudaEventCreateWithFlags(&rfork, cudaEventDisableTiming));
-            for (int i = 0; i < kResStreams; ++i) {
+        return FW_OK;
+    }
+    // The first `count` streams of resident launches (slots 0 .. count-1 use no
+    // others).  No more than are used: live streams slow the creation of any
+    // problem in the process, by 0.5 us each (with 33 batches of 2 problems
+    // alive 1.1 ms, and 1.6 when each held 32 streams).
+    fw_status res_streams(int count) {
+        if (!rfork) FW_CUDA(cudaEventCreateWithFlags(&rfork, cudaEventDisableTiming));
+        for (int i = 0; i < count; ++i) {
+            if (!rstream[i])
                 FW_CUDA(cudaStreamCreateWithFlags(&rstream[i], cudaStreamNonBlocking));
-                FW_CUDA(cudaEventCreateWithFlags(&rjoin[i], cudaEventDisableTiming));
-            }
+            if (!rjoin[i]) FW_CUDA(cudaEventCreateWithFlags(&rjoin[i], cudaEventDisableTiming));
         }
         return FW_OK;
     }
