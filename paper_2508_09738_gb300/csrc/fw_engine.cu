@@ -855,6 +855,8 @@ public:
 
     fw_status get_U(int s, double* out) {
         const ProbLayout& lay = slots[size_t(s)].lay;
+        if (lay.n * lay.K < kHostRowsMax)
+            return soa_to_host(slots[size_t(s)].pd.U, te, lay.n, lay.npad, lay.K, out, stream);
         Temps t(stream);
         void* scratch = nullptr;
         const size_t row = sizeof(double) * size_t(lay.K);

@@ -282,6 +282,8 @@ static fw_status status_of(const ProbState& st) {
 // d_tmp, or a few MB of the pool when the array is d_tmp itself.
 static fw_status copy_soa_to_host(fw_seg* h, const void* dev, double* out) {
     const ProbLayout& lay = h->lay;
+    if (lay.n * lay.K < kHostRowsMax)
+        return soa_to_host(dev, h->ops->elem(), lay.n, lay.npad, lay.K, out, h->stream);
     size_t bytes = h->ops->elem() * size_t(lay.npad) * size_t(lay.K);
     void* scratch = h->d_tmp;
     Temps t(h->stream);

@@ -514,6 +514,19 @@ private:
     std::vector<std::thread> th_;
 };
 
+fw_status soa_to_host(const void* X, size_t te, int64_t n, int64_t npad, int K, double* out,
+                      cudaStream_t s) {
+    std::vector<unsigned char> tmp(te * size_t(npad) * size_t(K));
+    FW_CUDA(cudaMemcpyAsync(tmp.data(), X, tmp.size(), cudaMemcpyDeviceToHost, s));
+    FW_CUDA(cudaStreamSynchronize(s));
+    const float* f = reinterpret_cast<const float*>(tmp.data());
+    const double* d = reinterpret_cast<const double*>(tmp.data());
+    for (int64_t i = 0; i < n; ++i)
+        for (int k = 0; k < K; ++k)
+            out[i * K + k] = te == 4 ? double(f[k * npad + i]) : d[k * npad + i];
+    return FW_OK;
+}
+
 fw_status rowmajor_to_host(Ops* ops, const void* X, int64_t n, int64_t npad, int K, double* out,
                            void* scratch, size_t bytes, cudaStream_t s) {
     PageToucher touch(out, sizeof(double) * size_t(n) * size_t(K));

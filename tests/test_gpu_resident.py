@@ -138,3 +138,24 @@ def test_oneshot_on_a_resident_problem():
             B.Segmenter(g, eps=0.1, omega0=1e5, index_width=32) as b:
         assert np.array_equal(a.oneshot()[0], b.oneshot()[0])
         assert a.solve().gap == b.solve().gap
+
+
+@pytest.mark.parametrize("weights", ["f32", "f64"])
+@pytest.mark.parametrize("n,K", [(33, 3), (16383, 4), (16384, 4), (16385, 4), (9362, 7), (9363, 7)])
+def test_read_out_around_the_host_line(n, K, weights):
+    """An iterate read back is the one written, exactly, on both sides of the
+    line between the read-out on the host (fewer than 65,536 values) and the
+    one on the device."""
+    i = np.arange(n)
+    rows = np.stack([(i - 1) % n, (i + 1) % n], 1)
+    rows.sort(axis=1)
+    g = W.Graph(n=n, row_ptr=np.arange(0, 2 * n + 1, 2, dtype=np.int32),
+                col=rows.ravel().astype(np.int32), w=np.ones(2 * n), K=K,
+                labels=np.where(i < K, i, -1).astype(np.int32), truth=(i % K).astype(np.int32))
+    rng = np.random.default_rng(5)
+    U = rng.integers(1, 64, (n, K)).astype(np.float64)
+    U[:, 0] += 4096 - U.sum(1)
+    U /= 4096.0     # multiples of 2^-12: exact in either type, rows sum to 1
+    with B.Segmenter(g, weight_dtype=weights) as s:
+        s.set_U(U)
+        assert np.array_equal(s.U(), U)
