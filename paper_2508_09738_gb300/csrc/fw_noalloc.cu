@@ -20,8 +20,8 @@
 //
 // Set-up: the first call on each device, with that device current, looks the
 // scratch array up with cudaGetSymbolAddress (which may load the module's
-// device data) and caches the address together with the identity of the
-// current CUDA context.  A later call in another context of that device (for
+// device data), sets the energy kernel's shared-memory limit, and caches the
+// address together with the identity of the current CUDA context.  A later call in another context of that device (for
 // instance after cudaDeviceReset) looks the address up again.  Make the first
 // call on a device before any stream capture.
 //
@@ -104,9 +104,14 @@ __device__ __forceinline__ double na_row_energy(int K, const double* __restrict_
 constexpr int kNaChunk = 256;
 // Dynamic shared memory of one warp: the chunk's weights and columns, the
 // rows' products.
-__host__ __device__ inline size_t na_warp_smem(int K) {
+__host__ __device__ constexpr size_t na_warp_smem(int K) {
     return size_t(kNaChunk) * (sizeof(double) + sizeof(int32_t)) + size_t(32) * K * sizeof(double);
 }
+constexpr int kNaMaxK = 32;
+// A block's, for the limit that k_na_energy is given (88 KB).  It is the same
+// for every K: what a kernel gets without asking, 48 KB, counts its 3,168
+// static bytes too and ends at K = 10.
+constexpr size_t kNaSmemMax = (kBlock / 32) * na_warp_smem(kNaMaxK);
 
 // Per row i (FP64): 1/2 sum_k u_ik (L u)_ik + 1/eps sum_k u_ik (1 - u_ik)
 // + 1/2 omega_i sum_k (uhat_ik - u_ik)^2, with (L u)_ik = u_ik - sum_j
@@ -258,7 +263,7 @@ unsigned long long current_ctx_id() {
 }
 
 // Device address of this device's scratch array, looked up once per device
-// and context.
+// and context, together with the energy kernel's shared-memory limit.
 fw_status na_scratch(void** out) {
     int dev = 0;
     FW_CUDA(cudaGetDevice(&dev));
@@ -275,6 +280,8 @@ fw_status na_scratch(void** out) {
         void* p = nullptr;
         const cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(g_noalloc_scratch)");
+        FW_CUDA(cudaFuncSetAttribute(k_na_energy, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     int(kNaSmemMax)));
         c.ptr = p;
         c.ctx = ctx;
     }
@@ -305,7 +312,7 @@ extern "C" fw_status fw_energy_noalloc(int64_t n, int32_t K, const int32_t* row_
                   std::to_string(kNaMaxN) + " rows");
         return FW_ERR_UNSUPPORTED;
     }
-    if (K < 2 || K > 32) return na_invalid("fw_energy_noalloc: K must be in [2, 32]");
+    if (K < 2 || K > kNaMaxK) return na_invalid("fw_energy_noalloc: K must be in [2, 32]");
     if (nnz < 0 || nnz >= (int64_t(1) << 31))
         return na_invalid("fw_energy_noalloc: nnz must be in [0, 2^31)");
     if (!row_ptr_dev || !U_dev || (nnz > 0 && (!col_dev || !w_dev)))
@@ -332,9 +339,6 @@ extern "C" fw_status fw_energy_noalloc(int64_t n, int32_t K, const int32_t* row_
     k_na_degrees<<<blocks, kBlock, 0, s>>>(n, nnz, row_ptr_dev, col_dev, w_dev, deg, acc);
     FW_CUDA(cudaGetLastError());
     const size_t smem = size_t(kBlock / 32) * na_warp_smem(K);
-    if (smem > 48 * 1024)   // K > 12: beyond what a kernel gets without asking
-        FW_CUDA(cudaFuncSetAttribute(k_na_energy, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     int(smem)));
     k_na_energy<<<blocks, kBlock, smem, s>>>(n, nnz, K, row_ptr_dev, col_dev, w_dev, deg, U_dev,
                                           ldu, labels_dev, std::isinf(eps) ? 0.0 : 1.0 / eps,
                                           omega0, laplacian == FW_LAPLACIAN_COMB ? 1 : 0, acc);
