@@ -301,7 +301,8 @@ typedef struct fw_batch_opts {
     int32_t weight_dtype;      /* FW_WEIGHTS_*, shared by every problem */
     int32_t blocks_per_sm;     /* 0: autotune (cached) */
     int32_t schedule;          /* FW_SCHED_* (AUTO: autotuned) */
-    int32_t iters_per_launch;  /* -1: autotune; 0: every iteration in one launch */
+    int32_t iters_per_launch;  /* -1: autotune; 0: every iteration in one launch (of problems
+                                  that the resident kernel takes, 4,096 a launch) */
     int32_t use_graph;         /* FW_GRAPH_* (default FW_GRAPH_REQUIRED) */
     int32_t spin_budget_ms;    /* bound on one grid-barrier wait */
     int32_t test_barrier_extra;/* test hook, keep 0: the barrier also waits for this many
@@ -346,7 +347,7 @@ typedef struct fw_batch fw_batch;
  * summed, so a batch equals single solves bit for bit when those use the
  * same lanes_per_row (fw_batch_info reports it).  When the resident kernel
  * takes every problem, nothing is timed: per-item schedule, each problem's own
- * lanes, all iterations in one launch.  The choice is cached in
+ * lanes, all iterations in one launch (4,096 at most).  The choice is cached in
  * tune_cache under a signature of the device and the batch's sizes. */
 fw_status fw_batch_default_opts(fw_batch_opts *opts);
 

@@ -13,6 +13,10 @@ namespace fw {
 constexpr int kResThreads = 512;
 constexpr int kResWarps = kResThreads / 32;
 constexpr int kResRing = 32;                      // iterations between statistics
+// Most iterations of one launch: a launch cannot be interrupted (this many
+// take a few tens of ms at most), and the arrival count of the grid barrier
+// (two per block and iteration) stays far below 2^32.
+constexpr int kResIters = 4096;
 constexpr int kResTilesPerLayer = kResThreads / kBlock;   // row tiles per layer of a block
 constexpr int kResMaxCluster = 16;
 constexpr int kResMaxGrid = 160;                  // blocks of a grid group
@@ -266,7 +270,7 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target) {
         for (;;) {
             uint32_t v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if (v >= target) break;
+            if (int32_t(v - target) >= 0) break;
             const unsigned long long t = globaltimer_ns();
             if (!t0) t0 = t;
             else if (t - t0 > kMbarWaitNs) {
@@ -1151,9 +1155,10 @@ inline cudaError_t res_build(ResKern* k, const ResArgs& a, ResPlan& p, cudaStrea
     if (e == cudaSuccess) k->sliced(p, chunks);
     return e;
 }
-// Enqueue up to `iters` iterations.
+// Enqueue up to `iters` iterations, and no more than kResIters and one last
+// evaluation: callers with more to do launch again.
 inline cudaError_t res_launch(ResKern* k, ResArgs a, const ResPlan& p, int iters, cudaStream_t s) {
-    a.iters = iters;
+    a.iters = std::min(iters, kResIters + 1);
     const cudaError_t e =
         a.cluster ? cudaSuccess : cudaMemsetAsync(a.bar, 0, sizeof(uint32_t), s);
     return e == cudaSuccess ? k->launch(a, p, s) : e;

@@ -105,9 +105,6 @@ struct fw_seg {
     }
 };
 
-// Iterations of one resident launch (a few tens of ms at most).
-constexpr int kResIters = 4096;
-
 static fw_status launch_check(const char* what) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, what);
