@@ -86,7 +86,8 @@ typedef struct fw_seg_opts {
                                  |j - i| < 2^15, as in pixel grids; else 32-bit) or 32 */
     int32_t class_table;      /* FW_TABLE_*: pass B reads the 4-bit classes from a copy in
                                  shared memory (same results; see below) */
-    int32_t reserved;         /* 0 */
+    int32_t test_barrier_extra; /* test hook, keep 0: waits inside the resident kernel are
+                                 for this much more that never arrives, so they run out */
     void *cuda_stream;        /* cudaStream_t for all work; NULL: the handle makes one */
 } fw_seg_opts;
 
@@ -156,7 +157,8 @@ fw_status fw_seg_create(fw_seg **out, int64_t n, const int32_t *row_ptr_host,
  * refresh_every > 0, or on a stream that cannot be captured, the host checks
  * the state after every launch.  Both forms give the same bits.  The stream
  * is synchronised on return.  FW_ERR_TIMEOUT: a wait inside the resident
- * kernel ran out of its 2 s. */
+ * kernel ran out of its 2 s; U is undefined until fw_seg_reset or
+ * fw_seg_set_U. */
 fw_status fw_seg_solve(fw_seg *h, fw_seg_stats *stats);
 
 /* Run at most `iters` iterations (fewer if the stop rule holds first) and
@@ -272,8 +274,8 @@ void fw_seg_destroy(fw_seg *h);
  * are bitwise the same as when it is solved alone (by fw_seg_* or in any
  * other batch) with the same lanes per row.  Each problem stops on its own
  * stop rule; later launches skip it.  Waits at the persistent kernel's grid
- * barrier are bounded by spin_budget_ms: a wait that runs out ends the launch
- * with FW_ERR_TIMEOUT instead of hanging.
+ * barrier and inside resident launches are bounded by spin_budget_ms: a wait
+ * that runs out ends the launch with FW_ERR_TIMEOUT instead of hanging.
  * ---------------------------------------------------------------------- */
 
 /* A graph on the host (see fw_seg_create for the CSR conventions). */
@@ -304,8 +306,8 @@ typedef struct fw_batch_opts {
     int32_t iters_per_launch;  /* -1: autotune; 0: every iteration in one launch (of problems
                                   that the resident kernel takes, 4,096 a launch) */
     int32_t use_graph;         /* FW_GRAPH_* (default FW_GRAPH_REQUIRED) */
-    int32_t spin_budget_ms;    /* bound on one grid-barrier wait */
-    int32_t test_barrier_extra;/* test hook, keep 0: the barrier also waits for this many
+    int32_t spin_budget_ms;    /* bound on one wait between a launch's blocks */
+    int32_t test_barrier_extra;/* test hook, keep 0: blocks also wait for this many
                                   blocks that never arrive, so every wait runs out */
     int32_t lanes_per_row;     /* -1: autotune; 0: each problem's own count (from its
                                   options, else its mean degree); else 1,2,4,..,32 for
@@ -400,7 +402,7 @@ typedef struct fw_srv_opts {
     int32_t iters_per_epoch;
     int32_t blocks_per_sm;     /* 0: largest co-resident grid */
     int32_t schedule;          /* FW_SCHED_* (default and AUTO: per-item launches) */
-    int32_t spin_budget_ms;
+    int32_t spin_budget_ms;    /* bound on one wait between a launch's blocks */
     int32_t reserved;
     void *cuda_stream;         /* stream of the epochs; NULL: the server makes one */
 } fw_srv_opts;

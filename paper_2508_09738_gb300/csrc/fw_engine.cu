@@ -182,7 +182,8 @@ public:
     bool res_outside = false;                    // slices may come from the library's pool
     int res_share = 0;                           // ResKern::plan
     bool crowded = false;                        // serving: other requests wait or run
-    long long budget = 0;
+    long long budget = 0;                        // cycles of one persistent-kernel wait
+    unsigned long long wait_ns = 0;              // the same bound for a resident launch
     cudaGraphExec_t graph = nullptr;
     int graph_iters = -1;
     bool work_dirty = true;
@@ -276,6 +277,7 @@ public:
         FW_CUDA(cudaDeviceGetAttribute(&clock_khz, cudaDevAttrClockRate, dev));
         if (clock_khz <= 0) clock_khz = 2100000;
         budget = (long long)std::max(spin_ms, 1) * (long long)clock_khz;
+        wait_ns = (unsigned long long)std::max(spin_ms, 1) * 1000000ull;
         set_grid(blocks_per_sm > 0 ? blocks_per_sm : occ,
                  (sched == FW_SCHED_STATIC || sched == FW_SCHED_ITEMS) ? sched : FW_SCHED_DYNAMIC);
         return FW_OK;
@@ -419,7 +421,8 @@ public:
             if (off == SIZE_MAX) return FW_OK;
             m = pool + off;
         }
-        sl.rargs = res_args(p, sl.pd, d_state + s, m);
+        sl.rargs = res_args(p, sl.pd, d_state + s, m, wait_ns,
+                            std::max(expect_extra, sl.opts.test_barrier_extra));
         sl.roff = off;
         sl.rmem = outside;
         sl.rbytes = need;

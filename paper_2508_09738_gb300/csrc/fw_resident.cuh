@@ -72,7 +72,8 @@ struct ResArgs {
     int32_t group;           // blocks that work on the problem: the cluster, or the grid
     int32_t cluster;         // 1: the group is a thread-block cluster, 0: the whole grid
     int32_t iters;           // iterations of this launch
-    int32_t pad_;
+    int32_t expect_extra;    // test hook: every wait is for this much that never arrives
+    unsigned long long wait_ns;   // bound of one wait inside the kernel
     uint32_t* bar;           // grid group: arrivals, zero at launch
     ResSlot* slots;          // grid group: [kNumR][group]
 };
@@ -240,8 +241,10 @@ __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
-// mbar_wait with the acquire scope that st_async from other blocks needs.
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
+// mbar_wait with the acquire scope that st_async from other blocks needs,
+// bounded by `limit` ns.
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity,
+                                                  unsigned long long limit) {
     uint32_t ok = 0;
     unsigned long long t0 = 0;
     for (;;) {
@@ -255,13 +258,14 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
         if (ok) return true;
         const unsigned long long t = globaltimer_ns();
         if (!t0) t0 = t;
-        else if (t - t0 > kMbarWaitNs) return false;
+        else if (t - t0 > limit) return false;
     }
 }
 
 // Barrier over the grid: arrival count with release / acquire at GPU scope,
-// the wait bounded in time (kMbarWaitNs).  False when it ran out.
-__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target) {
+// the wait bounded by `limit` ns.  False when it ran out.
+__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target,
+                                             unsigned long long limit) {
     __syncthreads();
     bool late = false;
     if (threadIdx.x == 0) {
@@ -273,7 +277,7 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target) {
             if (int32_t(v - target) >= 0) break;
             const unsigned long long t = globaltimer_ns();
             if (!t0) t0 = t;
-            else if (t - t0 > kMbarWaitNs) {
+            else if (t - t0 > limit) {
                 late = true;
                 break;
             }
@@ -623,7 +627,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
     for (int it = 0;;) {
         if (multi && tid == 0) {
             const int others = pd.ntiles * (kBlock / 32) - nu;
-            mbar_expect_tx(&bars[0], uint32_t(others) * (WIDE ? 16u : 32u));
+            mbar_expect_tx(&bars[0], uint32_t(others) * (WIDE ? 16u : 32u) +
+                                         uint32_t(a.expect_extra) * 16u);
             mbar_expect_tx(&bars[1], uint32_t(a.group - 1) * kNumR * 16u);
         }
         // ---------------------------------------------------------- phase A
@@ -761,10 +766,11 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
         if (!SHARED && chunks > 1) Q.load(col0, val0, 1);
         bool alive = true;
         if (a.cluster) {
-            const bool got = !multi || mbar_wait_cluster(&bars[0], uint32_t(it & 1));
+            const bool got = !multi || mbar_wait_cluster(&bars[0], uint32_t(it & 1), a.wait_ns);
             alive = !__syncthreads_or(!got);
         } else {
-            alive = grid_barrier(a.bar, target += uint32_t(a.group));
+            target += uint32_t(a.group);
+            alive = grid_barrier(a.bar, target + uint32_t(a.expect_extra), a.wait_ns);
             if (!WIDE) {
                 const uint4* src = reinterpret_cast<const uint4*>(pd.choice + sp.first);
                 for (int i = tid; i < sp.window / 16; i += kResThreads) {
@@ -964,7 +970,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
             if (warp == 0) {
                 // lane (p, q): quantity q of the blocks p, p + 4, ...
                 const int q = lane & 7, p = lane >> 3;
-                alive = !multi || mbar_wait_cluster(&bars[1], uint32_t(it & 1));
+                alive = !multi || mbar_wait_cluster(&bars[1], uint32_t(it & 1), a.wait_ns);
                 alive = __all_sync(0xffffffffu, alive);
                 unsigned long long lo = 0ull, hi = 0ull;
                 bool bad = false;
@@ -981,7 +987,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
                 __syncwarp();
             }
         } else {
-            alive = grid_barrier(a.bar, target += uint32_t(a.group));
+            target += uint32_t(a.group);
+            alive = grid_barrier(a.bar, target + uint32_t(a.expect_extra), a.wait_ns);
             if (warp < kNumR) {
                 unsigned long long lo = 0ull, hi = 0ull;
                 bool bad = false;
@@ -1121,9 +1128,12 @@ inline size_t res_bytes(const ResPlan& p) {
            res_up(size_t(p.entries) * p.welem);
 }
 // The launch parameters (but the iteration count) with those arrays at m.
-inline ResArgs res_args(const ResPlan& p, const ProbDesc& pd, ProbState* st, char* m) {
+inline ResArgs res_args(const ResPlan& p, const ProbDesc& pd, ProbState* st, char* m,
+                        unsigned long long wait_ns, int expect_extra) {
     ResArgs a{};
     a.state = st;
+    a.wait_ns = wait_ns;
+    a.expect_extra = std::max(expect_extra, 0);
     a.group = p.group;
     a.cluster = p.cluster;
     a.p.pd = pd;

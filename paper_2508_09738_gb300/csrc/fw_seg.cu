@@ -200,7 +200,7 @@ static fw_status plan_resident(fw_seg* h) {
         return FW_OK;
     char* m = nullptr;
     if (h->alloc(&m, res_bytes(p)) != FW_OK) return FW_OK;
-    h->res_args = res_args(p, h->pd, h->st, m);
+    h->res_args = res_args(p, h->pd, h->st, m, kMbarWaitNs, h->opts.test_barrier_extra);
     FW_CUDA(res_build(h->res.get(), h->res_args, p, h->stream));
     h->res_plan = p;
     return FW_OK;

@@ -1,5 +1,7 @@
 """Launches of the resident kernel: their length, their bounded waits, and
 what a caller learns when one runs out (GPU)."""
+import time
+
 import numpy as np
 import pytest
 
@@ -30,3 +32,43 @@ def test_batch_launches_hold_at_most_4096_iterations(per):
         sb = b.solve()[0]
         assert (sb.iters, sb.gap, sb.objective, sb.launches) == (9000, st.gap, st.objective, 3)
         assert np.array_equal(b.U(0), U)
+
+
+# a cluster's exchange, a grid's barrier
+@pytest.mark.parametrize("n", [3001, 30_001])
+def test_wait_that_runs_out_in_a_handle(n):
+    """Blocks that wait for more than ever arrives give up after 2 s: the
+    solve reports it, nothing hangs, and a reset makes the handle usable."""
+    g = W.blobs_knn(n=n, K=5, seed=3, label_frac=0.02)
+    with B.Segmenter(g, max_iters=20, class_table="off") as s:
+        want = s.step(20)
+        U = s.U()
+    with B.Segmenter(g, max_iters=20, test_barrier_extra=1) as s:
+        t0 = time.time()
+        with pytest.raises(B.FwError) as e:
+            s.solve()
+        assert e.value.status == B.FW_ERR_TIMEOUT
+        assert 1.0 < time.time() - t0 < 10.0
+        s.reset()
+        st = s.step(20)          # the launches of the two passes have no such waits
+        assert (st.gap, st.objective) == (want.gap, want.objective)
+        assert np.array_equal(s.U(), U)
+
+
+@pytest.mark.parametrize("n", [3001, 30_001])
+def test_wait_that_runs_out_in_a_server(n):
+    """spin_budget_ms bounds the waits of served resident launches; only the
+    request concerned fails."""
+    g = W.blobs_knn(n=n, K=5, seed=3, label_frac=0.02)
+    with B.Segmenter(g, max_iters=20) as s:
+        s.solve()
+        lab = s.labels()
+    with B.Server(hbm_budget_bytes=1 << 30, max_slots=4, max_K=8, spin_budget_ms=20) as srv:
+        t0 = time.time()
+        bad = srv.submit(g, max_iters=20, test_barrier_extra=1)
+        good = srv.submit(g, max_iters=20)
+        assert srv.wait(bad, g.n, timeout_ms=30_000)[0] == B.FW_ERR_TIMEOUT
+        assert time.time() - t0 < 1.5
+        rc, l, _ = srv.wait(good, g.n, timeout_ms=30_000)
+        assert rc == B.FW_NOT_CONVERGED and np.array_equal(l, lab)
+        assert srv.info().failed == 1
