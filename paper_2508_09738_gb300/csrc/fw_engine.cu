@@ -666,6 +666,7 @@ public:
         FW_CUDA(cudaStreamSynchronize(stream));
         FW_CUDA(cudaMemcpy(h_state, d_state, sizeof(ProbState) * slots.size(),
                            cudaMemcpyDeviceToHost));
+        for (int s = 0; s < nslots(); ++s) settle(h_state[s]);
         return FW_OK;
     }
 
@@ -713,6 +714,7 @@ public:
                 if (e == cudaErrorNotReady) break;
                 FW_CUDA(e);
                 h_state[s] = h_rring[i];
+                settle(h_state[s]);
                 sl.rhead ^= 1;
                 --sl.rqueued;
                 sl.rturn = ++rturns;
@@ -831,6 +833,7 @@ public:
             set_error("grid barrier wait ran out of its budget");
             return FW_ERR_TIMEOUT;
         }
+        for (int s = 0; s < nslots(); ++s) settle(h_state[s]);
         return FW_OK;
     }
 
@@ -1259,10 +1262,13 @@ fw_status fw_batch_solve(fw_batch* b, fw_seg_stats* stats) {
     for (int p = 0; p < b->P; ++p) {
         const ProbState& st = e.h_state[p];
         if (stats) fill_stats_from(st, stats + p, b->launches, ms);
-        if (st.status == FW_ERR_NUMERIC) worst = FW_ERR_NUMERIC;
+        // errors before the iteration cap; of two kinds of error the timeout,
+        // which leaves the problem's iterate undefined
+        if (st.status < 0) worst = std::min(worst, fw_status(st.status));
         else if (st.status == FW_NOT_CONVERGED && worst == FW_OK) worst = FW_NOT_CONVERGED;
     }
     if (worst == FW_ERR_NUMERIC) set_error("non-finite FW gap or curvature in a problem");
+    else if (worst == FW_ERR_TIMEOUT) set_error(kTimeoutText);
     return worst;
 }
 

@@ -99,6 +99,15 @@ public:
 // NULL when no resident kernel is compiled for K classes.
 ResKern* make_res(int weight_dtype, int K);
 
+// A state as copied from the device.  `err` says that a wait ran out in some
+// block; the decision of a block that saw none may have been stored beside it.
+inline void settle(ProbState& s) {
+    if (!s.err) return;
+    s.done = 1;
+    s.status = FW_ERR_TIMEOUT;
+}
+constexpr const char* kTimeoutText = "a wait between the blocks of a launch ran out of its budget";
+
 // Non-template kernels (defined in fw_seg.cu).
 __global__ void k_validate(int64_t n, const int32_t* rp, const int32_t* col, const double* w,
                            double* deg, int* err, int* band);

@@ -1081,7 +1081,10 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
     }
 
     __syncthreads();
-    if (s_fail) {   // a wait ran out: every block leaves, nothing is written back
+    // A wait ran out: this block writes no row back.  Another may have finished
+    // its last exchange and store its rows and the decision: `err`, which only
+    // a restart clears, then overrules them (settle).
+    if (s_fail) {
         if (tid == 0) {
             atomicExch(&st->err, 1);
             st->status = -7;   // FW_ERR_TIMEOUT

@@ -115,6 +115,7 @@ static fw_status read_state(fw_seg* h) {
     FW_CUDA(cudaMemcpyAsync(h->h_state, h->st, sizeof(ProbState), cudaMemcpyDeviceToHost,
                             h->stream));
     FW_CUDA(cudaStreamSynchronize(h->stream));
+    settle(*h->h_state);
     return FW_OK;
 }
 
@@ -272,6 +273,7 @@ static fw_status status_of(const ProbState& st) {
         set_error("non-finite FW gap or curvature");
         return FW_ERR_NUMERIC;
     }
+    if (st.status == FW_ERR_TIMEOUT) set_error(kTimeoutText);
     return fw_status(st.status);
 }
 

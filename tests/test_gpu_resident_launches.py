@@ -72,3 +72,30 @@ def test_wait_that_runs_out_in_a_server(n):
         rc, l, _ = srv.wait(good, g.n, timeout_ms=30_000)
         assert rc == B.FW_NOT_CONVERGED and np.array_equal(l, lab)
         assert srv.info().failed == 1
+
+
+@pytest.mark.parametrize("graph", ["required", "off"])
+@pytest.mark.parametrize("n", [3001, 30_001])
+def test_wait_that_runs_out_in_a_batch(n, graph):
+    """A batch does not report success for a problem whose launch gave up,
+    whatever the others' statuses are, and says which kind of error it was."""
+    g = W.blobs_knn(n=n, K=5, seed=3, label_frac=0.02)
+    ok = W.blobs_knn(n=500, K=3, seed=4)
+    opts = [B.fw_seg_default_opts(max_iters=20), B.fw_seg_default_opts(max_iters=20,
+                                                                       test_barrier_extra=1),
+            B.fw_seg_default_opts(max_iters=0)]
+    with B.Batch([ok, g, ok], opts, schedule="items", lanes_per_row=0, blocks_per_sm=1,
+                 iters_per_launch=0, spin_budget_ms=20, use_graph=graph) as b:
+        t0 = time.time()
+        with pytest.raises(B.FwError) as e:
+            b.solve()
+        assert time.time() - t0 < 1.5
+        assert e.value.status == B.FW_ERR_TIMEOUT and "wait" in str(e.value)
+        with B.Segmenter(ok, max_iters=20) as s:
+            s.solve()
+            assert np.array_equal(b.U(0), s.U())
+    with B.Batch([ok, g], B.fw_seg_default_opts(max_iters=20), schedule="items", lanes_per_row=0,
+                 blocks_per_sm=1, iters_per_launch=0, spin_budget_ms=20, test_barrier_extra=1) as b:
+        with pytest.raises(B.FwError) as e:
+            b.solve()
+        assert e.value.status == B.FW_ERR_TIMEOUT
