@@ -148,8 +148,11 @@ fw_status fw_seg_create(fw_seg **out, int64_t n, const int32_t *row_ptr_host,
  * Execution: problems of up to 311,296 rows and K <= 16 whose state fits the
  * chip (class_table left at FW_TABLE_AUTO) run in one launch of the resident
  * kernel: U and L U stay in registers from the first iteration to the last,
- * on one thread-block cluster or on a cooperative grid of one block per SM at
- * most.  Others run as a CUDA graph of iters_per_launch iterations
+ * on one thread-block cluster of at most 16 blocks or on a grid of one block
+ * per SM at most.  Such a block needs an SM to itself, all of them at once.
+ * A grid that finds other kernels on its SMs leaves again after 0.2 ms, the
+ * solve goes on with iters_per_launch iterations of the form below, and tries
+ * again; a cluster waits for its SMs.  Others run as a CUDA graph of iters_per_launch iterations
  * (2 kernels each, the step decision of each iteration taken at the start of
  * the next one, one finishing kernel per graph), launched repeatedly with one
  * launch queued ahead of the host's state check; fewer than iters_per_launch
@@ -266,7 +269,9 @@ void fw_seg_destroy(fw_seg *h);
  * offsets) and iterate together, from a captured CUDA graph, in one of two
  * schedules (FW_SCHED_*): per-item launches, where the problems that the
  * resident kernel of fw_seg_solve takes run in one such launch each, beside
- * each other, and each iteration of the rest is one
+ * each other (a launch starts when it has an SM for each of its blocks, so
+ * it waits for kernels of other streams that hold them), and each iteration
+ * of the rest is one
  * launch of pass A over the row tiles of every live problem and one of pass B
  * (the kernel boundaries are the barriers); or a cooperative persistent
  * kernel: phase A, grid barrier, phase B, grid barrier, per iteration.  Each

@@ -74,7 +74,11 @@ struct ResArgs {
     int32_t iters;           // iterations of this launch
     int32_t expect_extra;    // test hook: every wait is for this much that never arrives
     unsigned long long wait_ns;   // bound of one wait inside the kernel
-    uint32_t* bar;           // grid group: arrivals, zero at launch
+    // Grid group, > 0: an ordinary launch whose blocks first meet, for at most
+    // this long; if some find no SM meanwhile, all leave and the state says so
+    // (unstarted).  0: a cooperative launch, which starts when every block can.
+    unsigned long long meet_ns;
+    uint32_t* bar;           // grid group: arrivals, blocks that met; zero at launch
     ResSlot* slots;          // grid group: [kNumR][group]
 };
 
@@ -284,6 +288,36 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target,
         }
     }
     return !__syncthreads_or(late);
+}
+
+// Whether all blocks of an ordinary grid launch are on the device: each has
+// added itself to *word, and they wait for the last one for at most `limit`
+// ns.  The block that gives up first sets the top bit in exchange for a count
+// below `group`: a word holds either the bit or the full count, never both in
+// doubt, so all blocks leave, late ones included, or all go on (and then
+// they are resident together, and their barriers can be met).
+__device__ __forceinline__ bool grid_meet(uint32_t* word, uint32_t group, unsigned long long limit,
+                                          ProbState* st) {
+    int out = 0;
+    if (threadIdx.x == 0) {
+        unsigned long long t0 = 0;
+        for (;;) {
+            const uint32_t v = *reinterpret_cast<volatile uint32_t*>(word);
+            if (v >> 31) {
+                out = 1;
+                break;
+            }
+            if (v >= group) break;
+            const unsigned long long t = globaltimer_ns();
+            if (!t0) t0 = t;
+            else if (t - t0 > limit && atomicCAS(word, v, v | 0x80000000u) == v) {
+                st->unstarted = 1;
+                out = 1;
+                break;
+            }
+        }
+    }
+    return !__syncthreads_or(out);
 }
 
 // ------------------------------------------------------------------ warps
@@ -528,6 +562,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
     }
     __syncthreads();
     if (s_done) return;   // the same in every block of the group
+    if (a.meet_ns && tid == 0) atomicAdd(a.bar + 1, 1u);   // see grid_meet
     const int K = EXACT ? KMAX : pd.K, n = pd.n, L = pd.lanes;
     const int64_t np = pd.npad;
     const int layers = s_rp.layers;
@@ -622,6 +657,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
     val0 += (size_t(before) * 32 + lane) * 4;
     uint32_t target = 0;
     if (a.cluster) cluster_barrier();   // every block's shared memory can be written
+    // nothing but loads so far: without its blocks the launch leaves no trace
+    if (a.meet_ns && !grid_meet(a.bar + 1, uint32_t(a.group), a.meet_ns, st)) return;
     __syncthreads();
 
     for (int it = 0;;) {
@@ -1173,7 +1210,7 @@ inline cudaError_t res_build(ResKern* k, const ResArgs& a, ResPlan& p, cudaStrea
 inline cudaError_t res_launch(ResKern* k, ResArgs a, const ResPlan& p, int iters, cudaStream_t s) {
     a.iters = std::min(iters, kResIters + 1);
     const cudaError_t e =
-        a.cluster ? cudaSuccess : cudaMemsetAsync(a.bar, 0, sizeof(uint32_t), s);
+        a.cluster ? cudaSuccess : cudaMemsetAsync(a.bar, 0, 2 * sizeof(uint32_t), s);
     return e == cudaSuccess ? k->launch(a, p, s) : e;
 }
 
@@ -1209,6 +1246,8 @@ public:
             if (ct <= kResMaxCluster && attempt(pd, nt, ct, 1, p, maxlen, nnz_pad)) return true;
             if (nt <= sms && attempt(pd, nt, nt, 0, p, maxlen, nnz_pad)) return true;
         }
+        // All SMs, though fewer would do for the fullest block's tiles: 131 and 146
+        // blocks in place of 152 took 1 to 2% more (sbm200k, 613 x 487 image).
         const int c = std::min(kResMaxCluster, cluster_of(pairs)), g = std::min(sms, pairs);
         // A cluster exchanges in 400 cycles what the grid barrier takes 2,300
         // for, but has 16 SMs: with more than two layers a block the grid's
@@ -1310,6 +1349,7 @@ public:
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         config(cfg, attr, p.group, p.cluster, p.smem, s);
+        if (a.meet_ns) cfg.numAttrs = 0;
         return with(p.form, [&](auto kern) { return cudaLaunchKernelEx(&cfg, kern, a); });
     }
 };

@@ -240,9 +240,20 @@ static fw_status plan_patterns(fw_seg* h) {
     return FW_OK;
 }
 
+// How long the blocks of a solve's resident grid wait for the last one (beside
+// nothing else they are there within a microsecond).  Longer, and beside a
+// kernel that keeps its SM the 32 iterations between two attempts (0.3 ms at
+// least) would not be most of the time; shorter, and it would give up where
+// the other kernel is about to end.
+constexpr unsigned long long kResMeetNs = 200000;
+
 // Up to `iters` iterations in one resident launch (it ends at the stop rule).
-static fw_status launch_resident(fw_seg* h, int iters) {
-    FW_CUDA(res_launch(h->res.get(), h->res_args, h->res_plan, iters, h->stream));
+// With `meet` a grid that cannot be on the device as a whole leaves again and
+// h_state->unstarted says so; otherwise the launch waits until it can.
+static fw_status launch_resident(fw_seg* h, int iters, bool meet) {
+    ResArgs a = h->res_args;
+    a.meet_ns = meet && !a.cluster ? kResMeetNs : 0;
+    FW_CUDA(res_launch(h->res.get(), a, h->res_plan, iters, h->stream));
     ++h->launches;
     return FW_OK;
 }
@@ -530,16 +541,23 @@ fw_status fw_seg_solve(fw_seg* h, fw_seg_stats* stats) {
         }
         if (queued) FW_TRY(read_state(h));   // the launch queued after the stop
     }
+    bool held = false;   // the last resident launch found too few free SMs
     while (!h->h_state->done) {
         if (R > 0 && h->h_state->iter - h->last_refresh >= R) FW_TRY(refresh_lu(h));
         const int remaining = h->opts.max_iters - h->h_state->iter;
-        if (h->res_plan.group > 0) {
+        if (h->res_plan.group > 0 && !held) {
             // the whole solve in one launch: its last evaluation meets the
             // iteration cap.  With refreshes, as many iterations at a time as
             // a graph holds.
             const int it = R > 0 && remaining >= m ? m : std::min(remaining, kResIters) + 1;
-            FW_TRY(launch_resident(h, it));
-        } else if (remaining >= m && h->graph) {
+            FW_TRY(launch_resident(h, it, true));
+            FW_TRY(read_state(h));
+            held = h->h_state->unstarted != 0;
+            if (held) FW_CUDA(cudaMemsetAsync(&h->st->unstarted, 0, sizeof(int32_t), h->stream));
+            continue;   // m iterations of the two passes, which share SMs, then again
+        }
+        held = false;
+        if (remaining >= m && h->graph) {
             FW_CUDA(cudaGraphLaunch(h->graph, h->stream));
             h->launches += graph_launches(m);
         } else {
@@ -596,7 +614,7 @@ fw_status fw_seg_profile(fw_seg* h, int32_t iters, double* ms_a, double* ms_b, d
     fw_status res = FW_OK;
     FW_TRY(time_enqueued(h, graph, [&] {
         if (h->res_plan.group > 0) {
-            res = launch_resident(h, m);
+            res = launch_resident(h, m, false);
             return;
         }
         for (int i = 0; i < m; ++i) {

@@ -121,6 +121,8 @@ struct ProbState {
     uint32_t cntF;       // flush tiles arrived
     int32_t cur;         // parity: step inputs in[cur]; bank of the pending totals
     int32_t cur_b;       // accumulator bank of the running iteration's pass B
+    int32_t unstarted;   // 1: a resident launch left without a change (ResArgs::meet_ns)
+    int32_t pad_;
     StepIn in[2];
 };
 

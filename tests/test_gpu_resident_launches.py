@@ -99,3 +99,30 @@ def test_wait_that_runs_out_in_a_batch(n, graph):
         with pytest.raises(B.FwError) as e:
             b.solve()
         assert e.value.status == B.FW_ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("opts", [{}, dict(refresh_every=8, iters_per_launch=8)])
+def test_solve_goes_on_beside_kernels_that_keep_their_sms(opts):
+    """A grid of resident blocks that cannot all be placed leaves without a
+    trace, and the solve goes on beside the other kernels: it ends long before
+    them, with the same bits as alone, and so does one under way when they end."""
+    torch = pytest.importorskip("torch")
+    g = W.voronoi_image(side=552, height=540, K=6, label_frac=0.01, seed=4)   # 1,165 tiles
+    kw = dict(max_iters=200, omega0=1e5, **opts)
+    others = [torch.cuda.Stream() for _ in range(16)]   # one block, one SM each
+    with B.Segmenter(g, **kw) as s:
+        alone = s.solve()
+        U = s.U()
+        for ms in (300, 3):
+            s.reset()
+            torch.cuda.synchronize()
+            t0 = time.time()
+            for o in others:
+                with torch.cuda.stream(o):
+                    torch.cuda._sleep(int(ms * 2e6))
+            st = s.solve()
+            if ms == 300:
+                assert time.time() - t0 < 0.2
+            assert (st.gap, st.objective, st.iters) == (alone.gap, alone.objective, alone.iters)
+            assert np.array_equal(s.U(), U)
+            torch.cuda.synchronize()
