@@ -243,10 +243,10 @@ public:
         if (user_stream) {
             stream = static_cast<cudaStream_t>(user_stream);
         } else {
-            FW_CUDA(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
+            FW_CUDA(make_stream(&stream));
             own_stream = true;
         }
-        FW_CUDA(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
+        FW_CUDA(make_stream(&side));
         FW_TRY(dev_alloc((void**)&pool, pool_bytes));
         ra.init(pool_bytes);
         slots.assign(size_t(max_slots), Slot());
@@ -439,11 +439,11 @@ public:
     // problem in the process, by 0.5 us each (with 33 batches of 2 problems
     // alive 1.1 ms, and 1.6 when each held 32 streams).
     fw_status res_streams(int count) {
-        if (!rfork) FW_CUDA(cudaEventCreateWithFlags(&rfork, cudaEventDisableTiming));
+        if (!rfork) FW_CUDA(make_event(&rfork, cudaEventDisableTiming));
         for (int i = 0; i < count; ++i) {
             if (!rstream[i])
-                FW_CUDA(cudaStreamCreateWithFlags(&rstream[i], cudaStreamNonBlocking));
-            if (!rjoin[i]) FW_CUDA(cudaEventCreateWithFlags(&rjoin[i], cudaEventDisableTiming));
+                FW_CUDA(make_stream(&rstream[i]));
+            if (!rjoin[i]) FW_CUDA(make_event(&rjoin[i], cudaEventDisableTiming));
         }
         return FW_OK;
     }
@@ -676,14 +676,12 @@ public:
     // another or for the host.
     fw_status res_queue(const std::vector<int>& set, int iters) {
         if (ring_queued > 0) FW_TRY(drain_lone());
-        if (!h_rring) {
-            FW_CUDA(cudaMallocHost(&h_rring, 2 * slots.size() * sizeof(ProbState)));
-            for (size_t i = 0; i < 2 * slots.size(); ++i) {
-                cudaEvent_t ev = nullptr;
-                FW_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-                rring_ev.push_back(ev);
-            }
+        while (rring_ev.size() < 2 * slots.size()) {
+            cudaEvent_t ev = nullptr;
+            FW_CUDA(make_event(&ev, cudaEventDisableTiming));
+            rring_ev.push_back(ev);
         }
+        if (!h_rring) FW_CUDA(cudaMallocHost(&h_rring, 2 * slots.size() * sizeof(ProbState)));
         for (int round = 0; round < 2; ++round)
             for (int s : set) {
                 Slot& sl = slots[size_t(s)];
@@ -735,7 +733,7 @@ public:
         if (!h_ring) {
             FW_CUDA(cudaMallocHost(&h_ring, 2 * sizeof(ProbState)));
             for (cudaEvent_t& ev : ring_ev)
-                FW_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+                FW_CUDA(make_event(&ev, cudaEventDisableTiming));
         }
         if (!lone_graph || lone_slot != s || lone_iters != iters) {
             FW_TRY(drain_lone());
@@ -1032,8 +1030,8 @@ static fw_status batch_tune(fw_batch* b) {
     }
     const auto t0 = std::chrono::steady_clock::now();
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    FW_CUDA(cudaEventCreate(&ev0));
-    FW_CUDA(cudaEventCreate(&ev1));
+    FW_CUDA(make_event(&ev0, cudaEventDefault));
+    FW_CUDA(make_event(&ev1, cudaEventDefault));
     struct EvGuard {
         cudaEvent_t a, b;
         ~EvGuard() {
@@ -1238,8 +1236,8 @@ fw_status fw_batch_solve(fw_batch* b, fw_seg_stats* stats) {
     Engine& e = b->eng;
     const int per = b->ipl > 0 ? b->ipl : b->max_iters + 1;
     cudaEvent_t ev0, ev1;
-    FW_CUDA(cudaEventCreate(&ev0));
-    FW_CUDA(cudaEventCreate(&ev1));
+    FW_CUDA(make_event(&ev0, cudaEventDefault));
+    FW_CUDA(make_event(&ev1, cudaEventDefault));
     cudaEventRecord(ev0, e.stream);
     b->launches = 0;
     fw_status rc = FW_OK;

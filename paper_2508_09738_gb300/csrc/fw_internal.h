@@ -23,6 +23,19 @@ fw_status cuda_fail(cudaError_t e, const char* what);
         if (e_ != cudaSuccess) return fw::cuda_fail(e_, #call); \
     } while (0)
 
+// Streams and events as the runtime makes them, NULL when it cannot: what a
+// failed call leaves in the handle is not one to wait for or destroy.
+inline cudaError_t make_stream(cudaStream_t* s) {
+    const cudaError_t e = cudaStreamCreateWithFlags(s, cudaStreamNonBlocking);
+    if (e != cudaSuccess) *s = nullptr;
+    return e;
+}
+inline cudaError_t make_event(cudaEvent_t* ev, unsigned flags) {
+    const cudaError_t e = cudaEventCreateWithFlags(ev, flags);
+    if (e != cudaSuccess) *ev = nullptr;
+    return e;
+}
+
 // Kernel launchers for one (iterate type, weight type, class bound) choice.
 // Every launcher takes the problem's descriptor (device pointers inside).
 class Ops {

@@ -463,7 +463,7 @@ fw_status fw_seg_create(fw_seg** out, int64_t n, const int32_t* row_ptr, const i
         if (o.cuda_stream) {
             h->stream = static_cast<cudaStream_t>(o.cuda_stream);
         } else {
-            FW_CUDA(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
+            FW_CUDA(make_stream(&h->stream));
             h->own_stream = true;
         }
         std::unique_ptr<Upload> up(new Upload(h->stream));
@@ -476,9 +476,9 @@ fw_status fw_seg_create(fw_seg** out, int64_t n, const int32_t* row_ptr, const i
         FW_CUDA(cudaMallocHost(&h->h_state, 3 * sizeof(ProbState)));
         h->h_ring = h->h_state + 1;
         for (cudaEvent_t& e : h->ring_ev)
-            FW_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        FW_CUDA(cudaEventCreate(&h->ev0));
-        FW_CUDA(cudaEventCreate(&h->ev1));
+            FW_CUDA(make_event(&e, cudaEventDisableTiming));
+        FW_CUDA(make_event(&h->ev0, cudaEventDefault));
+        FW_CUDA(make_event(&h->ev1, cudaEventDefault));
         const size_t te = h->ops->elem(), we = h->ops->welem();
         const bool comb = o.laplacian == FW_LAPLACIAN_COMB;
         const ProbLayout& lay = h->lay;
@@ -599,8 +599,8 @@ fw_status fw_seg_profile(fw_seg* h, int32_t iters, double* ms_a, double* ms_b, d
     const int m = iters;
     const bool graph = stream_capturable(h);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    FW_CUDA(cudaEventCreate(&e0));
-    FW_CUDA(cudaEventCreate(&e1));
+    FW_CUDA(make_event(&e0, cudaEventDefault));
+    FW_CUDA(make_event(&e1, cudaEventDefault));
     struct EvGuard {
         cudaEvent_t a, b;
         ~EvGuard() {
@@ -711,10 +711,10 @@ fw_status fw_seg_oneshot(fw_seg* h, int32_t* labels_host, double* ms) {
     // the call 145 instead of 205 (four parts: 10 more).
     const int n = h->pd.n;
     const int parts = labels_host && n >= (1 << 20) ? kCopyParts : 1;
-    if (parts > 1 && !h->copy_stream) {
-        FW_CUDA(cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking));
+    if (parts > 1) {
         for (cudaEvent_t& e : h->part_ev)
-            FW_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+            if (!e) FW_CUDA(make_event(&e, cudaEventDisableTiming));
+        if (!h->copy_stream) FW_CUDA(make_stream(&h->copy_stream));
     }
     auto cut = [n, parts](int i) { return int(int64_t(n) * i / parts) & ~(kBlock - 1); };
     auto enqueue = [&]() -> cudaError_t {

@@ -184,7 +184,10 @@ static thread_local std::string g_last_error;
 void set_error(const std::string& msg) { g_last_error = msg; }
 const char* last_error_text() { return g_last_error.c_str(); }
 
+// The runtime also keeps the error as the thread's last one; reported here, it
+// must not be taken for that of a later launch.
 fw_status cuda_fail(cudaError_t e, const char* what) {
+    cudaGetLastError();
     set_error(std::string(what) + ": " + cudaGetErrorString(e));
     return FW_ERR_CUDA;
 }
