@@ -537,8 +537,11 @@ public:
         if (n <= work_cap) return FW_OK;
         if (d_work) cudaFree(d_work);
         d_work = nullptr;
-        work_cap = std::max<size_t>(n, 2 * work_cap);
-        return dev_alloc((void**)&d_work, sizeof(int2) * work_cap);
+        const size_t cap = std::max<size_t>(n, 2 * work_cap);
+        work_cap = 0;
+        FW_TRY(dev_alloc((void**)&d_work, sizeof(int2) * cap));
+        work_cap = cap;
+        return FW_OK;
     }
 
     BatchArgs args(int nlive, int iters) const {
@@ -842,14 +845,19 @@ public:
         return collect();
     }
 
+    fw_status ensure_labels_cap(size_t n) {
+        if (n <= d_labels_cap) return FW_OK;
+        if (d_labels) cudaFree(d_labels);
+        d_labels = nullptr;
+        d_labels_cap = 0;
+        FW_TRY(dev_alloc((void**)&d_labels, 4 * n));
+        d_labels_cap = n;
+        return FW_OK;
+    }
+
     fw_status labels(int s, int32_t* out, cudaStream_t st) {
         const Slot& sl = slots[size_t(s)];
-        if (size_t(sl.lay.n) > d_labels_cap) {
-            if (d_labels) cudaFree(d_labels);
-            d_labels = nullptr;
-            d_labels_cap = size_t(sl.lay.n);
-            FW_TRY(dev_alloc((void**)&d_labels, 4 * d_labels_cap));
-        }
+        FW_TRY(ensure_labels_cap(size_t(sl.lay.n)));
         ops->labels(sl.pd, d_labels, st);
         FW_CUDA(cudaGetLastError());
         FW_CUDA(cudaMemcpyAsync(out, d_labels, 4 * size_t(sl.lay.n), cudaMemcpyDeviceToHost, st));
@@ -859,13 +867,12 @@ public:
 
     fw_status get_U(int s, double* out) {
         const ProbLayout& lay = slots[size_t(s)].lay;
-        if (lay.n * lay.K < kHostRowsMax)
-            return soa_to_host(slots[size_t(s)].pd.U, te, lay.n, lay.npad, lay.K, out, stream);
         Temps t(stream);
         void* scratch = nullptr;
         const size_t row = sizeof(double) * size_t(lay.K);
         const size_t bytes = std::max(row * kRmRows, std::min(row * size_t(lay.n), size_t(8) << 20));
-        FW_TRY(t.get(&scratch, bytes));
+        if (lay.n * lay.K < kHostRowsMax || t.get(&scratch, bytes) != FW_OK)
+            return soa_to_host(slots[size_t(s)].pd.U, te, lay.n, lay.npad, lay.K, out, stream);
         return rowmajor_to_host(ops.get(), slots[size_t(s)].pd.U, lay.n, lay.npad, lay.K, out,
                                 scratch, bytes, stream);
     }
@@ -1215,6 +1222,15 @@ fw_status fw_batch_create(fw_batch** out, int32_t P, const fw_graph* graphs,
                 layers += (l.ntiles + kResTilesPerLayer - 1) / kResTilesPerLayer;
             e.res_share = int(std::min<int64_t>((layers + e.sms - 1) / e.sms, 4));
             e.res_outside = true;
+            // what solves and read-outs allocate comes before the slices, which
+            // are taken only if there is room
+            size_t items = 0, rows = 0;
+            for (const ProbLayout& l : lays) {
+                items += size_t(l.ntiles);
+                rows = std::max(rows, size_t(l.n));
+            }
+            FW_TRY(e.ensure_work_cap(items));
+            FW_TRY(e.ensure_labels_cap(rows));
             for (int p = 0; p < P; ++p) FW_TRY(e.plan_res(p));
         }
         b->ipl = std::max(0, b->bo.iters_per_launch);

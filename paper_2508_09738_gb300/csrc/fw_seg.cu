@@ -300,7 +300,8 @@ static fw_status copy_soa_to_host(fw_seg* h, const void* dev, double* out) {
     const size_t least = sizeof(double) * kRmRows * size_t(lay.K);
     if (dev == h->d_tmp || bytes < least) {
         bytes = std::max(least, std::min(2 * bytes, size_t(8) << 20));
-        FW_TRY(t.get(&scratch, bytes));
+        if (t.get(&scratch, bytes) != FW_OK)   // a full device: as for small arrays
+            return soa_to_host(dev, h->ops->elem(), lay.n, lay.npad, lay.K, out, h->stream);
     }
     return rowmajor_to_host(h->ops.get(), dev, lay.n, lay.npad, lay.K, out, scratch, bytes,
                             h->stream);

@@ -54,3 +54,30 @@ except B.FwError:
     assert np.array_equal(s.grad()[0], G)
 assert failed > 0
 """)
+
+
+def test_read_outs_need_no_device_memory():
+    """With the library's own reserve used up as well, U and the gradient come
+    back through the host."""
+    run("""
+def ring(n, K):
+    i = np.arange(n)
+    rows = np.stack([(i - 1) % n, (i + 1) % n], 1)
+    rows.sort(axis=1)
+    return W.Graph(n=n, row_ptr=np.arange(0, 2 * n + 1, 2, dtype=np.int32),
+                   col=rows.ravel().astype(np.int32), w=np.ones(2 * n), K=K,
+                   labels=np.where(i < K, i, -1).astype(np.int32), truth=(i % K).astype(np.int32))
+
+handles = []
+stream = torch.cuda.default_stream().cuda_stream or 2     # 2: the per-thread default stream
+for n in (3_000_000, 300_000, 30_000, 3_000, 300):
+    gr = ring(n, 16)
+    try:
+        while len(handles) < 2000:
+            handles.append(B.Segmenter(gr, cuda_stream=stream))
+    except B.FwError:
+        pass
+assert len(handles) < 2000
+assert np.array_equal(b.U(0), U) and np.array_equal(b.labels(0), lab)
+assert np.array_equal(s.grad()[0], G)
+""")
