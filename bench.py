@@ -128,24 +128,6 @@ def column_bytes(g) -> int:
     return 4 if far else 2
 
 
-def reads_patterns(g, forms, tbytes=4, class_table="auto") -> bool:
-    """Whether pass B and the one-shot pass take one pattern byte per row in
-    place of row offsets and columns: regular grids with at most 64 distinct
-    rows of 5 to 8 entries, K <= 8, an FP32 iterate, one lane per row, and more
-    rows than the resident kernel takes (mirrors the library's rule)."""
-    d = np.diff(g.row_ptr).astype(np.int64)
-    if (not forms or class_table != "auto" or tbytes != 4 or g.K > 8 or g.n <= 311_296
-            or forms.get("class_table") or forms.get("lanes_per_row") != 1
-            or forms.get("index_width") != 16 or not 4 < d.max() <= 8 or g.nnz < 5 * g.n
-            or 8 * g.n > 1.02 * ((d + 3) // 4 * 4).sum()):
-        return False
-    rows = np.repeat(np.arange(g.n, dtype=np.int64), d)
-    at = np.arange(g.nnz, dtype=np.int64) - np.repeat(g.row_ptr[:-1].astype(np.int64), d)
-    off = np.zeros((g.n, 8), dtype=np.int16)
-    off[rows, at] = g.col.astype(np.int64) - rows
-    return len(np.unique(off.view("V16").ravel())) <= 64
-
-
 def bytes_per_unit(n, nnz, K, wbytes, tbytes=4, cbytes=4, patterns=False):
     """Algorithmic bytes of one FW iteration (the method's minimum: U and L U
     read and written, the CSR once, row_ptr, choice and fidelity bytes) and of
@@ -162,9 +144,9 @@ def bytes_per_unit(n, nnz, K, wbytes, tbytes=4, cbytes=4, patterns=False):
 
 
 # the sources that define and instantiate the profiled kernels (pass A,
-# pass B, finish, one-shot); host-only set-up and driver code is not included
+# pass B, finish, one-shot, resident); host-only set-up and driver code is not included
 KERNEL_SOURCES = ("fw_types.h", "fw_step.cuh", "fw_device.cuh", "fw_kernels.cuh", "fw_ops.cuh",
-                  "fw_ops_f32.cu", "fw_ops_bf16.cu", "fw_ops_f64.cu")
+                  "fw_resident.cuh", "fw_ops_f32.cu", "fw_ops_bf16.cu", "fw_ops_f64.cu")
 
 
 def source_hash() -> str:
@@ -476,7 +458,10 @@ def run_batched(args, rank, world, local, emit=True):
         "oracle_sample": sample,
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"], "traffic": None,
-                     "kernel": ("k_itemA + k_itemB" if info.get("schedule") == 3 else "k_persistent"),
+                     "kernel": ("k_persistent" if info.get("schedule") != 3 else
+                                "k_resident" if info.get("resident") == P else
+                                "k_itemA + k_itemB" if not info.get("resident") else
+                                "k_resident, k_itemA + k_itemB"),
                      "peak_source": peaks["source"],
                      "algorithmic_bytes": "sum over problems of iteration bytes x iterations; "
                                           "whole solves timed (all of the batch's kernels)"},
@@ -653,7 +638,8 @@ def run_oneshot(args, rank, world, local):
         st = seg.solve()
         gfw_ms.append(st.ms)
     lab_gfw = seg.labels()
-    pat = reads_patterns(g, seg.forms().as_dict(), 8 if weights == "f64" else 4)
+    pat = seg.forms().solve == B.SOLVE["patterns"]
+    kernel = "k_osfw_pat" if pat else "k_osfw"
     seg.close()
     wb = {"f32": 4, "bf16": 2, "f64": 8}[weights]
     index = g.n if pat else 4 * (g.n + 1) + column_bytes(g) * g.nnz
@@ -662,9 +648,9 @@ def run_oneshot(args, rank, world, local):
     peaks = load_peaks()
     achieved = nbytes / (mean_ms / 1000.0) / 1e9
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                "frac": achieved / peaks["hbm_gbs"], "traffic": ncu_traffic("k_osfw", name),
-                "kernel": "k_osfw", "peak_source": peaks["source"],
-                "algorithmic_bytes_per_launch": nbytes, "kernel_ms": {"k_osfw": mean_ms}}
+                "frac": achieved / peaks["hbm_gbs"], "traffic": ncu_traffic(kernel, name),
+                "kernel": kernel, "peak_source": peaks["source"],
+                "algorithmic_bytes_per_launch": nbytes, "kernel_ms": {kernel: mean_ms}}
     e2e = None
     if not args.no_e2e:
         def pinned(a):
@@ -780,29 +766,39 @@ def compare_golden(gold, labels, E_gpu, traj, truth):
     return d
 
 
-def roofline_of(prof, g, weights, workload, peaks, forms=None, class_table="auto"):
+def roofline_of(prof, g, weights, workload, peaks, forms):
+    """The kernel a solve spends most of its time in against the copy rate: of
+    the two passes the slower one, or the resident kernel (per iteration)."""
     wb = {"f32": 4, "bf16": 2, "f64": 8}[weights]
     tb = 8 if weights == "f64" else 4
-    pat = reads_patterns(g, forms, tb, class_table)
+    solve = {0: "passes", 1: "patterns", 2: "resident"}[forms["solve"]]
+    pat = solve == "patterns"
     by = bytes_per_unit(g.n, g.nnz, g.K, wb, tb, column_bytes(g), pat)
-    dom = "csr_pass" if prof["pass_b"] >= prof["pass_a"] else "row_pass"
-    dom_ms = prof["pass_b"] if dom == "csr_pass" else prof["pass_a"]
-    kernel = {"csr_pass": "k_passB", "row_pass": "k_passA"}[dom]
+    dom, kernel, dom_ms = (("iteration", "k_resident", prof["per_iter"]) if solve == "resident" else
+                           ("csr_pass", "k_passB", prof["pass_b"])
+                           if prof["pass_b"] >= prof["pass_a"] else
+                           ("row_pass", "k_passA", prof["pass_a"]))
     achieved = by[dom] / (dom_ms / 1000.0) / 1e9
     key = workload if weights == "f32" else f"{workload}_{weights}"
     return {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": achieved / peaks["hbm_gbs"], "traffic": ncu_traffic(kernel, key),
             "kernel": kernel, "peak_source": peaks["source"],
             "kernel_form": (("k_passB_tab (class table in shared memory)"
-                             if forms and forms.get("class_table") else
+                             if forms["class_table"] else
                              "k_passB_pat (row patterns)" if pat else "k_passB_lc / k_passB")
-                            if kernel == "k_passB" else "k_passA"),
-            "algorithmic_bytes_per_launch": by[dom],
-            "timing": "CUDA events on the solver's stream around a captured graph of "
+                            if kernel == "k_passB" else
+                            "k_resident (U and L U stay on the chip: the bytes are those of the "
+                            "method, not moved)" if solve == "resident" else "k_passA"),
+            ("algorithmic_bytes_per_iteration" if solve == "resident" else
+             "algorithmic_bytes_per_launch"): by[dom],
+            "timing": "CUDA events on the solver's stream around one launch of the iterations"
+                      if solve == "resident" else "CUDA events on the solver's stream around a captured graph of "
                       "back-to-back launches of the kernel" if prof["in_graph"] else
                       "CUDA events around back-to-back direct launches of the kernel",
-            "kernel_ms": {"k_passA": prof["pass_a"], "k_passB": prof["pass_b"],
-                          "k_finish": prof["finish"]}}, by
+            "kernel_ms": dict({"k_passA": prof["pass_a"], "k_passB": prof["pass_b"],
+                               "k_finish": prof["finish"]},
+                              **({"k_resident_per_iteration": prof["per_iter"]}
+                                 if solve == "resident" else {}))}, by
 
 
 def time_arm(args, B, torch, g, c, weights, iters, stream, flush, clocks, world, rank):
@@ -851,8 +847,7 @@ def time_arm(args, B, torch, g, c, weights, iters, stream, flush, clocks, world,
 
 def arm_record(args, arm, g, c, weights, iters, world, peaks):
     """The JSON fields of one timed weight dtype."""
-    roof, by = roofline_of(arm["prof"], g, weights, args.workload, peaks, arm.get("forms"),
-                           args.class_table)
+    roof, by = roofline_of(arm["prof"], g, weights, args.workload, peaks, arm["forms"])
     ms_step = 1000.0 * arm["t_s"] / args.steps
     rec = {"value": arm["value"], "unit": "iter/s", "weights": weights,
            "ms_per_step": ms_step, "solves_per_s": world * args.steps / arm["t_s"],

@@ -241,6 +241,11 @@ fw_status fw_seg_profile(fw_seg *h, int32_t iters, double *ms_row_pass, double *
 /* Statistics of the handle's current state. */
 fw_status fw_seg_get_stats(fw_seg *h, fw_seg_stats *stats);
 
+/* What fw_seg_solve launches: pass A and pass B; the same, with pass B (and
+ * the one-shot pass) reading one offset pattern per row in place of columns
+ * and row offsets (regular grids); or the resident kernel. */
+enum { FW_SOLVE_PASSES = 0, FW_SOLVE_PATTERNS = 1, FW_SOLVE_RESIDENT = 2 };
+
 /* The kernel forms create chose for the handle (host data only, no device
  * call): they change no result, only the speed.  FW_ERR_INVALID_ARG when h or
  * forms is NULL. */
@@ -252,7 +257,7 @@ typedef struct fw_seg_forms {
     int32_t tiles;           /* row tiles of the row passes */
     int32_t tile_rows;       /* rows per tile (a multiple of 256) */
     int32_t kmax;            /* class bound the kernels were compiled for (>= K) */
-    int32_t reserved;
+    int32_t solve;           /* FW_SOLVE_* */
 } fw_seg_forms;
 fw_status fw_seg_get_forms(fw_seg *h, fw_seg_forms *forms);
 
@@ -332,7 +337,7 @@ typedef struct fw_batch_info {
                                   own count from its mean degree */
     int32_t iters_per_launch;  /* 0: every iteration in one launch */
     int32_t graph_error;       /* cudaError_t of the last failed capture, 0 if none */
-    int32_t reserved;
+    int32_t resident;          /* problems that run in resident launches */
     double tune_ms;            /* time spent autotuning */
     size_t pool_bytes;         /* device bytes of the problem pool */
 } fw_batch_info;

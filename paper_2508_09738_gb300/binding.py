@@ -45,7 +45,7 @@ class fw_seg_opts(ctypes.Structure):
 class fw_seg_forms(ctypes.Structure):
     _fields_ = [("lanes_per_row", c_int32), ("index_width", c_int32), ("class_table", c_int32),
                 ("table_blocks", c_int32), ("tiles", c_int32), ("tile_rows", c_int32),
-                ("kmax", c_int32), ("reserved", c_int32)]
+                ("kmax", c_int32), ("solve", c_int32)]
 
     def as_dict(self):
         return {f: getattr(self, f) for f, _ in self._fields_}
@@ -78,7 +78,7 @@ class fw_batch_info(ctypes.Structure):
     _fields_ = [("grid", c_int32), ("blocks_per_sm", c_int32), ("schedule", c_int32),
                 ("graph_captured", c_int32), ("tuned", c_int32), ("kmax", c_int32),
                 ("lanes_per_row", c_int32), ("iters_per_launch", c_int32),
-                ("graph_error", c_int32), ("reserved", c_int32),
+                ("graph_error", c_int32), ("resident", c_int32),
                 ("tune_ms", c_double), ("pool_bytes", c_size_t)]
 
     def as_dict(self) -> dict:
@@ -105,6 +105,7 @@ class fw_srv_info(ctypes.Structure):
 
 SCHED = {"auto": 0, "static": 1, "dynamic": 2, "items": 3}
 TABLE = {"auto": 0, "off": 1, "on": 2}
+SOLVE = {"passes": 0, "patterns": 1, "resident": 2}
 GRAPH = {"off": 0, "required": 1, "preferred": 2}
 
 _lib = None

@@ -1317,7 +1317,9 @@ fw_status fw_batch_get_info(fw_batch* b, fw_batch_info* info) {
     info->lanes_per_row = b->eng.lanes_all;
     info->iters_per_launch = b->ipl;
     info->graph_error = b->eng.graph_error;
-    info->reserved = 0;
+    info->resident = 0;
+    for (const Slot& s : b->eng.slots)
+        info->resident += b->eng.schedule == FW_SCHED_ITEMS && s.res.group > 0 ? 1 : 0;
     info->tune_ms = b->tune_ms;
     info->pool_bytes = b->eng.ra.cap();
     return FW_OK;

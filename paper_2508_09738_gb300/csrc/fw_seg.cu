@@ -880,6 +880,9 @@ fw_status fw_seg_get_forms(fw_seg* h, fw_seg_forms* f) {
     f->tiles = h->pd.ntiles;
     f->tile_rows = h->pd.tile_rows;
     f->kmax = h->ops ? h->ops->kmax() : 0;
+    f->solve = h->res_plan.group > 0 ? FW_SOLVE_RESIDENT
+               : h->pd.pat           ? FW_SOLVE_PATTERNS
+                                     : FW_SOLVE_PASSES;
     return FW_OK;
 }
 
