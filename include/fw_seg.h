@@ -115,8 +115,8 @@ typedef struct fw_seg fw_seg;
  * the array plus the bins within one block's shared memory (n <= 280,574
  * for 8 < K <= 10 with 2 lanes), else the direct form runs.  Both forms give the
  * same bits.  FW_TABLE_OFF always runs the direct form.  Under either of the
- * two, fw_seg_solve runs that pass B also where it would run the resident
- * kernel under FW_TABLE_AUTO. */
+ * two, fw_seg_solve, batches and the server run pass A and pass B also where
+ * they would run the resident kernel under FW_TABLE_AUTO. */
 enum { FW_TABLE_AUTO = 0, FW_TABLE_OFF = 1, FW_TABLE_ON = 2 };
 
 /* Fill *opts with defaults: eps 50, omega0 1000 (the paper's network values,
@@ -275,8 +275,9 @@ void fw_seg_destroy(fw_seg *h);
  * schedules (FW_SCHED_*): per-item launches, where the problems that the
  * resident kernel of fw_seg_solve takes run in one such launch each, beside
  * each other (a launch starts when it has an SM for each of its blocks, so
- * it waits for kernels of other streams that hold them), and each iteration
- * of the rest is one
+ * it waits for kernels of other streams that hold them; a class_table option
+ * other than FW_TABLE_AUTO keeps a problem out), and each iteration of the
+ * rest is one
  * launch of pass A over the row tiles of every live problem and one of pass B
  * (the kernel boundaries are the barriers); or a cooperative persistent
  * kernel: phase A, grid barrier, phase B, grid barrier, per iteration.  Each

@@ -402,6 +402,7 @@ public:
     // library's pool.  Without room the slot runs as items.
     fw_status plan_res(int s) {
         Slot& sl = slots[size_t(s)];
+        if (sl.opts.class_table != FW_TABLE_AUTO) return FW_OK;   // as in a handle
         auto it = reskern.find(sl.lay.K);
         if (it == reskern.end())
             it = reskern.emplace(sl.lay.K, std::unique_ptr<ResKern>(make_res(wd, sl.lay.K))).first;
