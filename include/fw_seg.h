@@ -126,7 +126,9 @@ enum { FW_TABLE_AUTO = 0, FW_TABLE_OFF = 1, FW_TABLE_ON = 2 };
 fw_status fw_seg_default_opts(fw_seg_opts *opts);
 
 /* Device bytes a handle needs for a graph of n nodes, nnz stored entries and
- * K classes (peak during create), for admission control. */
+ * K classes (peak during create), for admission control.  Where there is more,
+ * the resident kernel's copy of a small graph may take up to 1 MB beyond it;
+ * without, the handle solves by pass A and pass B. */
 size_t fw_seg_footprint(int64_t n, int64_t nnz, int32_t K, int32_t weight_dtype);
 
 /* Create a solver for one graph (Sec. 1 graph, Sec. 2 fidelity data).
@@ -271,7 +273,8 @@ void fw_seg_destroy(fw_seg *h);
  * Batched solves: many independent problems iterated together.
  *
  * All problems of a batch live in one contiguous device pool (each at its own
- * offsets) and iterate together, from a captured CUDA graph, in one of two
+ * offsets; the resident kernel's copies of their graphs, taken while there is
+ * memory, lie outside it) and iterate together, from a captured CUDA graph, in one of two
  * schedules (FW_SCHED_*): per-item launches, where the problems that the
  * resident kernel of fw_seg_solve takes run in one such launch each, beside
  * each other (a launch starts when it has an SM for each of its blocks, so
@@ -340,7 +343,8 @@ typedef struct fw_batch_info {
     int32_t graph_error;       /* cudaError_t of the last failed capture, 0 if none */
     int32_t resident;          /* problems that run in resident launches */
     double tune_ms;            /* time spent autotuning */
-    size_t pool_bytes;         /* device bytes of the problem pool */
+    size_t pool_bytes;         /* device bytes of the problem pool and of the resident
+                                  kernel's copies of the graphs */
 } fw_batch_info;
 
 typedef struct fw_batch fw_batch;

@@ -1328,10 +1328,13 @@ fw_status fw_batch_get_info(fw_batch* b, fw_batch_info* info) {
     info->iters_per_launch = b->ipl;
     info->graph_error = b->eng.graph_error;
     info->resident = 0;
-    for (const Slot& s : b->eng.slots)
+    size_t slices = 0;
+    for (const Slot& s : b->eng.slots) {
         info->resident += b->eng.schedule == FW_SCHED_ITEMS && s.res.group > 0 ? 1 : 0;
+        slices += s.rmem ? s.rbytes : 0;
+    }
     info->tune_ms = b->tune_ms;
-    info->pool_bytes = b->eng.ra.cap();
+    info->pool_bytes = b->eng.ra.cap() + slices;
     return FW_OK;
 }
 

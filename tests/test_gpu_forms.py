@@ -41,3 +41,15 @@ def test_batch_counts_its_resident_problems():
                      blocks_per_sm=1, iters_per_launch=0) as b:
             b.solve()
             assert b.info().resident == want, schedule
+
+
+def test_batch_info_counts_the_slices():
+    """pool_bytes holds the resident kernel's copies of the graphs too: at
+    least a column and a weight for every entry."""
+    gs = [W.blobs_knn(n=4000, K=K, seed=K) for K in (3, 5, 8)]
+    got = {}
+    for table in ("auto", "off"):
+        with B.Batch(gs, B.fw_seg_default_opts(max_iters=5, class_table=table), schedule="items",
+                     lanes_per_row=0, blocks_per_sm=1, iters_per_launch=0) as b:
+            got[table] = b.info().pool_bytes
+    assert got["auto"] - got["off"] >= sum(g.nnz for g in gs) * (2 + 4)
