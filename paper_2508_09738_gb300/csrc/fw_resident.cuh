@@ -544,6 +544,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
     __shared__ __align__(16) ResSlot s_slot[kResMaxCluster][kNumR];
     __shared__ __align__(16) ResSlot s_ring[kResRing][kNumR];   // totals of iteration it % kResRing
     __shared__ __align__(16) T s_part[kNumR][R * kResWarps];
+    __shared__ __align__(16) uint4 s_note;      // from blocks without rows, never read
     __shared__ __align__(8) uint64_t bars[2];   // classes, totals from the cluster's blocks
     __shared__ int s_bad;                       // a total is not finite
     __shared__ T s_alpha;
@@ -664,10 +665,17 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
     for (int it = 0;;) {
         if (multi && tid == 0) {
             const int others = pd.ntiles * (kBlock / 32) - nu;
+            const int notes = max(a.group - pd.ntiles, 0) - (nu == 0 ? 1 : 0);
             mbar_expect_tx(&bars[0], uint32_t(others) * (WIDE ? 16u : 32u) +
-                                         uint32_t(a.expect_extra) * 16u);
+                                         uint32_t(notes + a.expect_extra) * 16u);
             mbar_expect_tx(&bars[1], uint32_t(a.group - 1) * kNumR * 16u);
         }
+        // A block's classes also say that it has read the last totals, so that
+        // the next may overwrite them.  A block without rows (fewer tiles than
+        // blocks, FP64) has none to send: it sends a note instead.
+        if (multi && nu == 0 && warp == 0 && lane < a.group && lane != rank)
+            st_async(map_rank(smem_u32(&s_note), uint32_t(lane)),
+                     map_rank(smem_u32(&bars[0]), uint32_t(lane)), make_uint4(0u, 0u, 0u, 0u));
         // ---------------------------------------------------------- phase A
 #pragma unroll
         for (int r = 0; r < R; ++r) {
