@@ -917,18 +917,20 @@ struct fw_batch {
 
 static std::string tune_signature(const fw_batch* b) {
     int64_t rows = 0, nnz = 0, tiles = 0;
+    int res = 0;   // with and without resident launches other choices are the best
     for (const Slot& s : b->eng.slots) {
         rows += s.lay.n;
         nnz += s.lay.nnz_pad;
         tiles += s.lay.ntiles;
+        res += s.res.group > 0 ? 1 : 0;
     }
     cudaDeviceProp p{};
     int dev = 0;
     cudaGetDevice(&dev);
     cudaGetDeviceProperties(&p, dev);
     char buf[512];
-    std::snprintf(buf, sizeof(buf), "v3|%s|wd%d|k%d|P%d|rows%lld|nnz%lld|tiles%lld|want%d%d%d%d",
-                  p.name, b->eng.wd, b->eng.kmax, b->P, (long long)rows, (long long)nnz,
+    std::snprintf(buf, sizeof(buf), "v4|%s|wd%d|k%d|P%d|res%d|rows%lld|nnz%lld|tiles%lld|want%d%d%d%d",
+                  p.name, b->eng.wd, b->eng.kmax, b->P, res, (long long)rows, (long long)nnz,
                   (long long)tiles, b->bo.blocks_per_sm, b->bo.schedule, b->bo.lanes_per_row,
                   b->bo.iters_per_launch);
     std::string s(buf);
