@@ -35,14 +35,14 @@ public:
         return (pd.tile_rows > kBlock ? max_stages<T, KMAX>() : 1) * 3 * size_t(kBlock) *
                size_t(pd.K) * sizeof(T);
     }
-    // f(the exact pass A of K classes), for K this class bound serves
+    // f(the exact pass A of K <= KMAX classes)
     template <typename F>
     static cudaError_t exactA(int K, F f) {
         if constexpr (kExactA) {
             switch (K) {
-                case 2: if constexpr (KMAX == 4) return f(k_passA_exact<T, 2>); break;
-                case 3: if constexpr (KMAX == 4) return f(k_passA_exact<T, 3>); break;
-                case 4: if constexpr (KMAX == 4) return f(k_passA_exact<T, 4>); break;
+                case 2: return f(k_passA_exact<T, 2>);
+                case 3: return f(k_passA_exact<T, 3>);
+                case 4: return f(k_passA_exact<T, 4>);
                 case 5: if constexpr (KMAX == 8) return f(k_passA_exact<T, 5>); break;
                 case 6: if constexpr (KMAX == 8) return f(k_passA_exact<T, 6>); break;
                 case 7: if constexpr (KMAX == 8) return f(k_passA_exact<T, 7>); break;
@@ -61,7 +61,8 @@ public:
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, int(smemA()));
             if (e != cudaSuccess) return e;
         } else {
-            for (int K = KMAX / 2 + (KMAX == 8); K <= KMAX; ++K) {
+            // four classes and fewer stay below 48 KB
+            for (int K = KMAX == 8 ? 5 : 2; K <= KMAX; ++K) {
                 e = exactA(K, [](auto kern) {
                     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 int(smemA()));
@@ -162,9 +163,9 @@ public:
         if constexpr (kPat) {
             if (pd.pat) {
                 switch (pd.K) {
-                    case 2: if constexpr (KMAX == 4) passB_pat<2>(pd, st, s); return;
-                    case 3: if constexpr (KMAX == 4) passB_pat<3>(pd, st, s); return;
-                    case 4: if constexpr (KMAX == 4) passB_pat<4>(pd, st, s); return;
+                    case 2: passB_pat<2>(pd, st, s); return;
+                    case 3: passB_pat<3>(pd, st, s); return;
+                    case 4: passB_pat<4>(pd, st, s); return;
                     case 5: if constexpr (KMAX == 8) passB_pat<5>(pd, st, s); return;
                     case 6: if constexpr (KMAX == 8) passB_pat<6>(pd, st, s); return;
                     case 7: if constexpr (KMAX == 8) passB_pat<7>(pd, st, s); return;
@@ -200,9 +201,9 @@ public:
         if constexpr (kPat) {
             if (pd.pat) {
                 switch (pd.K) {
-                    case 2: if constexpr (KMAX == 4) k_osfw_pat<WT, 2><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
-                    case 3: if constexpr (KMAX == 4) k_osfw_pat<WT, 3><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
-                    case 4: if constexpr (KMAX == 4) k_osfw_pat<WT, 4><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
+                    case 2: k_osfw_pat<WT, 2><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
+                    case 3: k_osfw_pat<WT, 3><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
+                    case 4: k_osfw_pat<WT, 4><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
                     case 5: if constexpr (KMAX == 8) k_osfw_pat<WT, 5><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
                     case 6: if constexpr (KMAX == 8) k_osfw_pat<WT, 6><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
                     case 7: if constexpr (KMAX == 8) k_osfw_pat<WT, 7><<<g, kBlock, 0, s>>>(pd, labels, first, last); return;
