@@ -1135,6 +1135,13 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
             st->status = -7;   // FW_ERR_TIMEOUT
             st->done = 1;
         }
+        // what other blocks have sent here, and nobody waits for now, arrives
+        // before this block lets the cluster end (a few microseconds at most)
+        if (a.cluster) {
+            const unsigned long long t0 = globaltimer_ns();
+            while (globaltimer_ns() - t0 < 100000ull) {
+            }
+        }
     } else {
         // ---- write the iterate back; the last evaluation's choice and L S with it
         T* __restrict__ Ub = static_cast<T*>(pd.U);
