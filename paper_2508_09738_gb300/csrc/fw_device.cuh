@@ -832,7 +832,7 @@ __device__ __forceinline__ void stage_issue(const ProbDesc& pd, int base, int ro
 
 // Pass A with the previous iteration's step decision fused in (ProbState):
 // when `fin`, the block decides on accumulator bank `cur` and in[cur] while
-// its first copies are in flight, and block 0 (`commit`) writes the result.
+// its first copies are in flight; a block without rows writes the result.
 struct FuseCtl {
     bool fin;
     const int* stop;        // shared memory: the decision stops the solve

@@ -49,7 +49,7 @@ __device__ __forceinline__ void passA_step(const ProbDesc& pd, ProbState* st, in
     __shared__ __align__(8) uint64_t bars[2];
     __shared__ T s_alpha;
     __shared__ int s_stop, s_done, s_cur;
-    // Block 0 of this launch may commit a stop (done = 1) while other blocks
+    // The committing block may store a stop (done = 1) while other blocks
     // start: one thread reads the flag (and the parity) and the whole block
     // follows it, so no block splits between leaving and waiting on the bulk
     // copies; that thread issues the copies as soon as it knows.

@@ -85,20 +85,20 @@ struct StepIn {
     int32_t iter, g0_set;
 };
 
-// Mutable per-problem state, in device memory.  The first block (iterate
-// fields) or the single finishing thread writes it; the next pass reads it.
+// Mutable per-problem state, in device memory.  One block of a pass (which
+// one: below) or k_finish's warp writes it; the next pass reads it.
 //
 // Step decisions.  Iteration t's totals complete when its pass B ends; the
 // stop test and the step length that follow from them are needed by pass A of
-// t+1.  Either a one-thread k_finish takes the decision between the passes,
+// t+1.  Either a one-warp k_finish takes the decision between the passes,
 // or (inside a captured graph) every block of pass A of t+1 takes the same
-// decision from the same totals and inputs, and only its first block writes
-// the result here.  So that no block reads a field another block of the same
+// decision from the same totals and inputs, and only a block that has no rows
+// (one more than the tiles) writes the result here.  So that no block reads a field another block of the same
 // pass writes, the inputs are kept twice (in[cur] is read, in[cur ^ 1]
 // written) and the totals alternate between the two accumulator banks:
 //   pass A (decision fused): reads bank cur and in[cur], accumulates into
-//                            bank cur ^ 1, block 0 writes in[cur ^ 1] and
-//                            cur_b = cur ^ 1;
+//                            bank cur ^ 1; the block without rows writes
+//                            in[cur ^ 1], block 0 cur_b = cur ^ 1;
 //   pass A (plain):          accumulates into bank cur, block 0 writes
 //                            cur_b = cur;
 //   pass B:                  accumulates into bank cur_b; block 0 sets
