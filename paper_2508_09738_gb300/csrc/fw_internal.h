@@ -191,6 +191,10 @@ struct Temps {
     }
 };
 
+// Whether the pages of a host buffer have been touched, by four of them (about
+// 1 us); false also when the system cannot say.
+bool pages_present(const void* p, size_t bytes);
+
 // Copy a class-major array X[K][npad] (n rows) to the host as row-major doubles;
 // `scratch` (device, `bytes` long) holds as many rows at a time as it can.
 // Waits for the stream.

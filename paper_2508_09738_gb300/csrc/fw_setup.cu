@@ -2,6 +2,7 @@
 // option and CSR checks, device layout, upload, validation, Laplacian
 // assembly (Sec. 1), U_0 = U_hat (Sec. 5.1), L U_0 and the initial state.
 #include <cuda_runtime.h>
+#include <sys/mman.h>
 #include <unistd.h>
 
 #include <algorithm>
@@ -486,6 +487,16 @@ fw_status pool_alloc(void** out, size_t bytes, cudaStream_t s) {
     return FW_OK;
 }
 
+
+bool pages_present(const void* p, size_t bytes) {
+    const uintptr_t page = uintptr_t(std::max<long>(sysconf(_SC_PAGESIZE), 4096));
+    for (size_t i = 1; i < 8; i += 2) {
+        const uintptr_t a = (reinterpret_cast<uintptr_t>(p) + bytes / 8 * i) & ~(page - 1);
+        unsigned char in = 0;
+        if (mincore(reinterpret_cast<void*>(a), page, &in) != 0 || !(in & 1)) return false;
+    }
+    return true;
+}
 
 // Write one byte of every page of an output buffer with a few threads, so that
 // the copy into it does not fault its pages one by one (134 MB of fresh pages:
