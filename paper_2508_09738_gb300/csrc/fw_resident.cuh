@@ -540,6 +540,9 @@ template <typename T, typename WT, int KMAX, bool EXACT, int FORM>
 __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_constant__ ResArgs a) {
     constexpr int R = res_layers<T, KMAX>();
     constexpr bool WIDE = FORM == kResWide, SHARED = FORM == kResShared;
+    // a cluster can have blocks without rows (plan(): FP64 alone takes more
+    // blocks than pairs of tiles rounded up to a power of two)
+    constexpr bool empties = sizeof(T) == 8;
     extern __shared__ __align__(128) unsigned char smraw[];
     __shared__ __align__(16) ResSlot s_slot[kResMaxCluster][kNumR];
     __shared__ __align__(16) ResSlot s_ring[kResRing][kNumR];   // totals of iteration it % kResRing
@@ -665,15 +668,15 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_consta
     for (int it = 0;;) {
         if (multi && tid == 0) {
             const int others = pd.ntiles * (kBlock / 32) - nu;
-            const int notes = max(a.group - pd.ntiles, 0) - (nu == 0 ? 1 : 0);
+            const int notes = empties ? max(a.group - pd.ntiles, 0) - (nu == 0 ? 1 : 0) : 0;
             mbar_expect_tx(&bars[0], uint32_t(others) * (WIDE ? 16u : 32u) +
                                          uint32_t(notes + a.expect_extra) * 16u);
             mbar_expect_tx(&bars[1], uint32_t(a.group - 1) * kNumR * 16u);
         }
         // A block's classes also say that it has read the last totals, so that
         // the next may overwrite them.  A block without rows (fewer tiles than
-        // blocks, FP64) has none to send: it sends a note instead.
-        if (multi && nu == 0 && warp == 0 && lane < a.group && lane != rank)
+        // blocks) has none to send: it sends a note instead.
+        if (empties && multi && nu == 0 && warp == 0 && lane < a.group && lane != rank)
             st_async(map_rank(smem_u32(&s_note), uint32_t(lane)),
                      map_rank(smem_u32(&bars[0]), uint32_t(lane)), make_uint4(0u, 0u, 0u, 0u));
         // ---------------------------------------------------------- phase A
