@@ -191,8 +191,8 @@ struct Temps {
     }
 };
 
-// Whether the pages of a host buffer have been touched, by four of them (about
-// 1 us); false also when the system cannot say.
+// Whether all pages of a host buffer have been touched; false also when the
+// system cannot say.
 bool pages_present(const void* p, size_t bytes);
 
 // Copy a class-major array X[K][npad] (n rows) to the host as row-major doubles;

@@ -490,41 +490,55 @@ fw_status pool_alloc(void** out, size_t bytes, cudaStream_t s) {
 
 bool pages_present(const void* p, size_t bytes) {
     const uintptr_t page = uintptr_t(std::max<long>(sysconf(_SC_PAGESIZE), 4096));
-    for (size_t i = 1; i < 8; i += 2) {
-        const uintptr_t a = (reinterpret_cast<uintptr_t>(p) + bytes / 8 * i) & ~(page - 1);
-        unsigned char in = 0;
-        if (mincore(reinterpret_cast<void*>(a), page, &in) != 0 || !(in & 1)) return false;
+    const uintptr_t end = reinterpret_cast<uintptr_t>(p) + bytes;
+    unsigned char in[1024];
+    for (uintptr_t a = reinterpret_cast<uintptr_t>(p) & ~(page - 1); a < end;) {
+        const size_t cnt = std::min<size_t>((end - a + page - 1) / page, sizeof(in));
+        if (mincore(reinterpret_cast<void*>(a), cnt * page, in) != 0) return false;
+        for (size_t i = 0; i < cnt; ++i)
+            if (!(in[i] & 1)) return false;
+        a += cnt * page;
     }
     return true;
 }
 
-// Write one byte of every page of an output buffer with a few threads, so that
-// the copy into it does not fault its pages one by one (134 MB of fresh pages:
-// 5 ms in the copy, 1.4 ms here).  Threads that cannot be started are skipped.
+// Write one byte of every page of an output buffer, so that the copy into it
+// does not fault its pages one by one: with a few threads from 16 MB on (134 MB
+// of fresh pages: 5 ms in the copy, 1.4 ms here; threads that cannot be started
+// are skipped), else in join(), where some are not there yet (read-outs into new
+// memory: 15 MB 0.9 to 8 ms, 0.7 to 0.8 here; 1.9 MB 0.36 ms, 0.14 here).
 class PageToucher {
 public:
-    PageToucher(void* p, size_t bytes) {
+    PageToucher(void* p, size_t bytes) : p_(static_cast<char*>(p)), bytes_(bytes) {
         if (bytes < (size_t(16) << 20)) return;
-        const size_t page = size_t(std::max<long>(sysconf(_SC_PAGESIZE), 4096));
         const size_t nt = std::min(8u, std::max(1u, std::thread::hardware_concurrency()));
-        char* const c = static_cast<char*>(p);
         try {
             th_.reserve(nt);
             for (size_t t = 0; t < nt; ++t)
-                th_.emplace_back([=] {
-                    for (size_t b = bytes * t / nt; b < bytes * (t + 1) / nt; b += page)
-                        reinterpret_cast<volatile char*>(c)[b] = 0;
-                });
+                th_.emplace_back([this, bytes, t, nt] { touch(bytes * t / nt, bytes * (t + 1) / nt); });
         } catch (...) {   // the threads that did start are joined
         }
+        bytes_ = 0;
     }
-    ~PageToucher() { join(); }
+    ~PageToucher() { finish(); }
     void join() {
-        for (auto& x : th_) x.join();
-        th_.clear();
+        finish();
+        if (bytes_ > 0 && !pages_present(p_, bytes_)) touch(0, bytes_);
+        bytes_ = 0;
     }
 
 private:
+    void finish() {
+        for (auto& x : th_) x.join();
+        th_.clear();
+    }
+    void touch(size_t from, size_t to) const {
+        const size_t page = size_t(std::max<long>(sysconf(_SC_PAGESIZE), 4096));
+        for (size_t b = from; b < to; b += page) reinterpret_cast<volatile char*>(p_)[b] = 0;
+        if (to > from) reinterpret_cast<volatile char*>(p_)[to - 1] = 0;
+    }
+    char* p_;
+    size_t bytes_;   // still to be touched in join()
     std::vector<std::thread> th_;
 };
 
