@@ -191,9 +191,8 @@ struct Temps {
     }
 };
 
-// Whether all pages of a host buffer have been touched; false also when the
-// system cannot say.
-bool pages_present(const void* p, size_t bytes);
+// Touch the pages of a host output buffer, unless all of them have been.
+void touch_pages(void* p, size_t bytes);
 
 // Copy a class-major array X[K][npad] (n rows) to the host as row-major doubles;
 // `scratch` (device, `bytes` long) holds as many rows at a time as it can.

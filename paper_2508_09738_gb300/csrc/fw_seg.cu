@@ -709,10 +709,10 @@ fw_status fw_seg_oneshot(fw_seg* h, int32_t* labels_host, double* ms) {
     // Large label arrays leave in parts, each copied (on a stream of the
     // handle's own, behind the part's kernel) while the next part is computed:
     // at 2048 x 2048 the copy takes 89 us, the kernel about 50 in two parts,
-    // the call 145 instead of 205 (four parts: 10 more).  Not into a buffer
-    // whose pages are yet to be touched (looked up while the kernels run):
-    // copied in parts they took 1.3 to 8 ms a call (which, differed from
-    // process to process), in one copy 0.8.
+    // the call 140 instead of 205 (four parts: 10 more).  A buffer's pages are
+    // touched before, while the kernels run: copies into new memory took 0.8 to
+    // 17 ms a call in one part and 1.1 to 17 in two (which, depended on how the
+    // memory came to be), 0.6 to 0.8 so.
     const int n = h->pd.n;
     const int parts = labels_host && n >= (1 << 20) ? kCopyParts : 1;
     if (parts > 1) {
@@ -729,11 +729,11 @@ fw_status fw_seg_oneshot(fw_seg* h, int32_t* labels_host, double* ms) {
             if (e == cudaSuccess && parts > 1) e = cudaEventRecord(h->part_ev[i], h->stream);
         }
         if (e == cudaSuccess) e = cudaEventRecord(h->ev1, h->stream);
-        const int copies = parts > 1 && pages_present(labels_host, 4 * size_t(n)) ? parts : 1;
-        for (int i = 0; i < copies && labels_host && e == cudaSuccess; ++i) {
-            const cudaStream_t s = copies > 1 ? h->copy_stream : h->stream;
-            const int r0 = cut(i), r1 = i + 1 < copies ? cut(i + 1) : n;
-            if (copies > 1) e = cudaStreamWaitEvent(s, h->part_ev[i], 0);
+        if (parts > 1 && e == cudaSuccess) touch_pages(labels_host, 4 * size_t(n));
+        for (int i = 0; i < parts && labels_host && e == cudaSuccess; ++i) {
+            const cudaStream_t s = parts > 1 ? h->copy_stream : h->stream;
+            const int r0 = cut(i), r1 = i + 1 < parts ? cut(i + 1) : n;
+            if (parts > 1) e = cudaStreamWaitEvent(s, h->part_ev[i], 0);
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(labels_host + r0, h->d_labels + r0, 4 * size_t(r1 - r0),
                                     cudaMemcpyDeviceToHost, s);

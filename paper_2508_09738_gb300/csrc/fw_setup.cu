@@ -488,7 +488,9 @@ fw_status pool_alloc(void** out, size_t bytes, cudaStream_t s) {
 }
 
 
-bool pages_present(const void* p, size_t bytes) {
+// Whether all pages of a host buffer have been touched; false also when the
+// system cannot say.
+static bool pages_present(const void* p, size_t bytes) {
     const uintptr_t page = uintptr_t(std::max<long>(sysconf(_SC_PAGESIZE), 4096));
     const uintptr_t end = reinterpret_cast<uintptr_t>(p) + bytes;
     unsigned char in[1024];
@@ -541,6 +543,12 @@ private:
     size_t bytes_;   // still to be touched in join()
     std::vector<std::thread> th_;
 };
+
+void touch_pages(void* p, size_t bytes) {
+    cudaPointerAttributes at{};   // a device address is left to the copy, which refuses it
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) cudaGetLastError();
+    if (at.type != cudaMemoryTypeDevice && !pages_present(p, bytes)) PageToucher(p, bytes).join();
+}
 
 fw_status soa_to_host(const void* X, size_t te, int64_t n, int64_t npad, int K, double* out,
                       cudaStream_t s) {

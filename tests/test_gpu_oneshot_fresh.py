@@ -19,8 +19,8 @@ def _built():
 
 def test_untouched_buffers_cost_one_copy():
     """What fw_seg_labels pays for such a buffer (a kernel, one copy and the
-    page faults in it) is what the one-shot call pays, beside its longer kernel
-    (0.1 ms); and the labels are those that touched buffers receive."""
+    page faults in it) is the most that the one-shot call pays, beside its longer
+    kernel (0.1 ms); and the labels are those that touched buffers receive."""
     g = W.voronoi_image(side=2048, height=2048, K=4, label_frac=0.01, seed=1)
     keep, ms = [], {}
     with B.Segmenter(g, eps=0.1, max_iters=2) as s:
