@@ -171,7 +171,7 @@ public:
     // slot s on stream s mod kResStreams.  30 k-NN problems (1,000 to 60,000
     // points, 200 iterations, BF16): 14.3 ms a batch with two launches per
     // iteration over all tiles, 10.1 with one resident launch each; a burst of
-    // 12 served requests 21.6 -> 16.2 ms.
+    // 12 served requests 21.6 -> 14.3 ms (with its later steps).
     std::map<int, std::unique_ptr<ResKern>> reskern;   // per class count
     cudaStream_t rstream[kResStreams] = {};
     cudaEvent_t rfork = nullptr, rjoin[kResStreams] = {};
